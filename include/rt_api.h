@@ -126,7 +126,17 @@ int rt_healpix_dirs(int nside, double* h_out);
  *     RT_MODE_F32_KAHAN, float64 for RT_MODE_FP64; fully written (rays from a
  *     source outside the domain get zeros and set RT_ERR_SOURCE_OUTSIDE).
  * The first call for a given nside on a device uploads its direction table
- * (an allocation); make that call outside CUDA graph capture. */
+ * (an allocation); make that call outside CUDA graph capture.
+ * On a full cube of equal-level leaves (32^3 or more), sources in consecutive
+ * leaves (Morton order), at least a sixteenth of them, that share one offset
+ * inside their leaf (leaf centres, for example) take no walk: every ray of a
+ * direction has the same steps, and the columns are summed from step tables
+ * and a row-ordered copy of the densities, bit for bit those of the walk.  The
+ * sources are checked on the device; those elsewhere (all, if over a sixteenth
+ * of them) are walked.  The handle keeps the tables and the copies (two of
+ * n_leaves x 1, 2, 4 or 8 values), allocated by the first such call and grown
+ * when a later one needs more; without memory for them, or on a stream under
+ * capture, every source is walked. */
 int rt_trace_columns(const rt_octree* tree, const double* d_src, int64_t n_src, int nside,
                      const void* d_dens, int n_species, int dens_dtype, int mode,
                      void* d_out, void* stream);
@@ -242,8 +252,8 @@ int rt_trace_paths(const rt_octree* tree, const double* d_src, int64_t n_src, in
  *       (leaf centres, for example), every ray of a direction takes the same
  *       steps and segment lengths, and each leaf's gradient is gathered by one
  *       thread from per-direction step tables: no atomics, and the same bits
- *       on every run (F32-Kahan: FP32 products with Kahan compensation, added
- *       once per leaf in FP64).  The sources are checked on the device; any
+ *       on every run (F32-Kahan: a Kahan sum of the FP32 products of each
+ *       direction, added once per leaf and direction in FP64).  The sources are checked on the device; any
  *       other call (and this one if the check fails) recomputes the paths
  *       and scatters with FP64 atomics, whose summation order is not fixed.
  *       The first gather on a handle allocates its step tables (kept by the
@@ -340,7 +350,9 @@ int rt_set_step_cap(rt_octree* tree, int64_t cap);
  * forward of rt_trace_columns on a full cube of equal-level leaves with FP32
  * densities of 1, 2, 4 or 8 species walks two rays per lane: its warps pop
  * one 64-source block and one direction group at a time, whatever
- * groups_per_pop says, and at most 3 of its blocks fit on an SM. */
+ * groups_per_pop says, and at most 3 of its blocks fit on an SM.  The form of
+ * rt_trace_columns and the adjoint that walks nothing has a launch shape of its
+ * own. */
 int rt_set_launch(int threads_per_block, int blocks_per_sm, int groups_per_pop);
 
 /* Caps the coarse-table level of later rt_build_octree calls (-1, the

@@ -214,6 +214,7 @@ void rt_destroy_octree(rt_octree* t)
     if (t->table) cudaFree(t->table);
     if (t->st) cudaFree(t->st);
     if (t->adj_tab) cudaFree(t->adj_tab);
+    if (t->fwd_tab && !t->fwd_tab_lent) cudaFree(t->fwd_tab);
     free(t);
 }
 
@@ -287,13 +288,18 @@ int rt::trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_sr
     a.dens_f64 = dens_dtype == RT_F64;
     a.out = d_out;
     cudaStream_t s = (cudaStream_t)stream;
-    if (check) {
-        const int cs = check_densities(d_dens, t->dev.n, n_species, a.dens_f64, 0, t->st, s);
-        if (cs != RT_OK) return cs;
-    }
     // (a general octree keeps one direction per pop: there the direction-major
     // sweep's L2 reuse of the walk outweighs the output's partial bursts)
     if (a.t.uniform_level >= 0) a.dgroup = output_dgroup(a.nd, n_species, mode);
+    // sources at one offset in consecutive leaves of a cube: no walk at all;
+    // the walk below then traces those the device finds elsewhere
+    bool beam = false;
+    st = launch_beam((rt_octree*)t, a, mode, false, check, s, &beam);
+    if (st != RT_OK) return st;
+    if (!beam && check) {
+        st = check_densities(d_dens, t->dev.n, n_species, a.dens_f64, 0, t->st, s);
+        if (st != RT_OK) return st;
+    }
     // leaf centres of a uniform cube share their exit sequences: two rays per
     // lane (FP32 densities with 1, 2, 4 or 8 species, direction-major order)
     a.pair = mode == RT_MODE_F32_KAHAN && a.t.uniform_level >= 0 && a.layout == 0 && !a.dens_f64 &&

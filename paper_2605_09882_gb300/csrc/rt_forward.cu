@@ -37,7 +37,8 @@ cudaError_t launch_forward(const TraceArgs& a, int mode, int block, int grid, cu
         case 8: k_trace_pair<8><<<grid, block, 0, s>>>(a); break;
         default: return cudaErrorInvalidValue;
         }
-        return cudaGetLastError();
+        if (!a.gate) return cudaGetLastError();
+        // then the sources the shared-offset form left out, one ray per lane
     }
     return dispatch<0>(a, mode, block, grid, s);
 }

@@ -29,7 +29,11 @@ int trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_src, i
 // argument checks and TraceArgs of the single-octree trace entry points
 int prepare_trace(const rt_octree* t, const double* d_src, int64_t n_src, int nside, int S, int mode,
                   TraceArgs& a, const char* who);
-// leaf-gather adjoint (rt_gather.cu): whether the call's shape admits it, and
+// shared-offset trace of a cube (rt_beam.cu): the scratch it needs (0: the
+// shape does not admit it) and its launch, with the density check if asked
+size_t beam_bytes(const rt_octree* t, int64_t n_src, int nd, int S, int mode);
+int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check, cudaStream_t s, bool* ran);
+// leaf-gather adjoint (rt_beam.cu): whether the call's shape admits it, and
 // its launch (source check, step tables, gather) on stream s
 bool gather_applies(const rt_octree* t, const TraceArgs& a);
 int launch_adjoint_gather(rt_octree* t, const TraceArgs& a, int mode, cudaStream_t s);

@@ -14,7 +14,7 @@ using namespace rt;
 
 namespace {
 
-enum { kKeys, kLevels, kDens, kSrc, kOut0, kOut1, kBufs };
+enum { kKeys, kLevels, kDens, kSrc, kOut0, kOut1, kRows, kBufs };
 
 struct Workspace {
     void* buf[kBufs] = {};
@@ -137,6 +137,17 @@ extern "C" int rt_trace_columns_host(const uint64_t* h_keys, const uint8_t* h_le
         return cuda_error(who);
     int st = rt_build_octree(keys, levels, n_leaves, h_extent, stream, &guard.tree);
     if (st != RT_OK) return st;
+    // scratch of the shared-offset trace, kept between calls (without it the
+    // handle of this call would allocate its own, or walk)
+    if (const size_t need = n_src ? beam_bytes(guard.tree, std::min(chunk, n_src), (int)nd, S, mode) : 0) {
+        const size_t had = w.cap[kRows];
+        if (reserve(w, kRows, need)) {
+            if (w.cap[kRows] != had) cudaMemsetAsync(w.buf[kRows], 0, 256, cs);  // no step tables in it yet
+            guard.tree->fwd_tab = w.buf[kRows];
+            guard.tree->fwd_tab_bytes = w.cap[kRows];
+        }
+        guard.tree->fwd_tab_lent = 1;
+    }
     // the source chunks follow on the upload stream, in order, under the
     // traces of the chunks before them
     for (int64_t c = 0; c < n_chunks; c++) {

@@ -71,7 +71,8 @@ struct TraceArgs {
     int batch;               // 32-ray groups per queue pop
     int layout;              // ray order: 0 direction-major (sources padded to 32), 1 source-major
     int dgroup;              // layout 0: directions per group (a power of two dividing nd; <= 1: one)
-    int pair;                // forward on a uniform cube: two rays per lane (k_trace_pair); n_src_pad % 64 == 0
+    int pair;                // forward on a uniform cube: two rays per lane (k_trace_pair; n_src_pad % 64 == 0),
+                             // k_trace then only for the sources the shared-offset form left out
     // path recording (KIND 3): per 32-ray group, segment k of lane i is entry
     // rec_off[g] + 32 k + i of rec_leaf / rec_ds
     const long long* rec_off;
@@ -82,9 +83,13 @@ struct TraceArgs {
     double epi_w[kMaxSpecies];
     double epi_a, epi_gamma;
     const double* epi_coef;
-    // adjoint scatter: runs only if *gate is nonzero (the leaf-gather form did
-    // not apply to this call); NULL: always runs
+    // runs only if *gate is nonzero (the shared-offset form launched before it
+    // did not apply to this call); NULL: always runs
     const int* gate;
+    // forward and epilogue: the sources the shared-offset form left out, walked
+    // when *gate is zero (NULL: none)
+    const uint32_t* rest;
+    const unsigned int* n_rest;
 };
 
 // Ray order of a trace: direction-major (32 neighbouring sources share a
@@ -114,5 +119,8 @@ struct rt_octree {
     int64_t default_cap;
     void* adj_tab;           // device, owned: step tables of the leaf-gather adjoint (grown on demand)
     size_t adj_tab_bytes;
+    void* fwd_tab;           // device: step tables and row-layout densities of the shared-offset trace
+    size_t fwd_tab_bytes;
+    int fwd_tab_lent;        // fwd_tab belongs to the caller that built the handle
     unsigned long long gen;  // build number, unique in the process (a reused address is another tree)
 };

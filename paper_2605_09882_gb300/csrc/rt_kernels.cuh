@@ -239,10 +239,15 @@ __global__ void __launch_bounds__(256, (MODE == RT_MODE_F32_KAHAN) ? (UNIFORM ? 
                                                                 : RT_MIN_BLOCKS)
 k_trace(const TraceArgs a)
 {
-    if (KIND == 2 && a.gate && *(volatile const int*)a.gate == 0) return;  // the leaf gather ran instead
+    // the shared-offset form ran before: only the sources it left out, if any
+    const bool rest = UNIFORM && a.gate && *(volatile const int*)a.gate == 0;
+    if (UNIFORM && a.pair && !rest) return;  // k_trace_pair traced every source
+    const unsigned n_rest = rest && a.n_rest ? *(volatile const unsigned*)a.n_rest : 0u;
+    if (rest && n_rest == 0u) return;
     if (MODE == RT_MODE_F32_KAHAN && !UNIFORM) fill_spread_table();
     const int lane = threadIdx.x & 31;
-    const unsigned long long total = (unsigned long long)(a.layout ? a.n_src : a.n_src_pad) * (unsigned long long)a.nd;
+    const unsigned long long rest_pad = (n_rest + 31u) & ~31u;
+    const unsigned long long total = (rest ? rest_pad : (unsigned long long)(a.layout ? a.n_src : a.n_src_pad)) * (unsigned long long)a.nd;
     const long long cap = a.t.step_cap;
     unsigned long long n_rays = 0, n_segs = 0, n_efb = 0, n_lfb = 0;
     for (;;) {
@@ -255,7 +260,12 @@ k_trace(const TraceArgs a)
             if (g0 >= total) break;
             int q;
             long long s;
-            if (a.layout == 0 && a.dgroup <= 1) {
+            if (rest) {
+                q = (int)(g0 / rest_pad);
+                const unsigned long long i = g0 - (unsigned long long)q * rest_pad + lane;
+                if (i >= n_rest) continue;
+                s = (long long)__ldg(a.rest + i);
+            } else if (a.layout == 0 && a.dgroup <= 1) {
                 q = (int)(g0 / (unsigned long long)a.n_src_pad);
                 s = (long long)(g0 - (unsigned long long)q * a.n_src_pad) + lane;
                 if (s >= a.n_src) continue;
@@ -369,6 +379,7 @@ __device__ __forceinline__ void store_cols(const TraceArgs& a, long long ray, co
 template <int SM>
 __global__ void __launch_bounds__(256, RT_MIN_BLOCKS_PAIR) k_trace_pair(const TraceArgs a)
 {
+    if (a.gate && *(volatile const int*)a.gate == 0) return;  // the shared-offset form ran instead
     const int lane = threadIdx.x & 31;
     const int D = a.dgroup > 1 ? a.dgroup : 1;
     const unsigned long long nb2 = (unsigned long long)a.n_src_pad >> 6;

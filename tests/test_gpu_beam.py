@@ -1,0 +1,111 @@
+"""Sources at one offset in consecutive leaves of a cube: the columns come from
+per-direction step tables instead of a walk, and must be bit for bit those of
+the walk, as must the statistics.
+
+The walk is what the same call does for fewer than a sixteenth of the leaves,
+so the reference traces the sources in slices."""
+import numpy as np
+import pytest
+
+import synth
+from tinytrees import uniform_octree
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rt():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2605_09882_gb300 as rt
+    return rt
+
+
+def _dev(a):
+    import torch
+    a = np.ascontiguousarray(a)
+    return torch.from_numpy(a.view(np.int64) if a.dtype == np.uint64 else a).cuda()
+
+
+def _stats(tree):
+    st = tree.stats()
+    assert st["status"] == 0, st
+    return st["rays"], st["segments"], st["exit_fallbacks"]
+
+
+def _sources(keys, lev, how, rng):
+    c = synth.leaf_centres(synth.Cloud(keys, lev, np.zeros((keys.shape[0], 1)), (1 << 21,) * 3))
+    n = c.shape[0]
+    h = 2.0 ** -int(lev[0])
+    if how == "offset":          # off the centre, off the depth-21 lattice
+        return c + (np.array([7 / 32, -11 / 32, 3 / 64]) + np.array([3, 5, -7]) * 2.0 ** -35) * h
+    if how == "range":           # part of the leaves: ragged, not aligned to a block of any kind
+        return c[n // 5 + 3:n // 2 + 18]
+    if how == "some_moved":      # some sources elsewhere, the first among them: the walk traces those
+        idx = np.concatenate([[0, 1, 33, n - 1], rng.integers(0, n, n // 40)])
+        c[idx] += (rng.random((idx.size, 3)) - 0.5) * 0.9 * h
+        return c
+    if how == "many_moved":      # too many: the walk traces all
+        idx = rng.integers(0, n, n // 4)
+        c[idx] += (rng.random((idx.size, 3)) - 0.5) * 0.9 * h
+        return c
+    if how == "last_place":      # one unit in the last place below the centre in some leaves
+        c[::11] = np.nextafter(c[::11], 0.0)
+        return c
+    return c
+
+
+@pytest.mark.parametrize("level,S,nside,dens,how", [
+    (5, 1, 1, "f32", "centres"), (5, 4, 2, "f32", "centres"), (5, 8, 1, "f64", "centres"), (5, 3, 1, "f32", "offset"),
+    (5, 2, 2, "f64", "range"), (6, 4, 1, "f32", "range"), (5, 4, 1, "f32", "some_moved"), (5, 2, 1, "f32", "many_moved"),
+    (6, 1, 2, "f32", "last_place"), (5, 5, 4, "f32", "centres")])
+@pytest.mark.parametrize("mode", ["f32k", "fp64"])
+def test_columns_equal_the_walk(rt, level, S, nside, dens, how, mode):
+    import torch
+    rng = np.random.default_rng(1200 + 10 * level + S)
+    keys, lev = uniform_octree(level)
+    src = _dev(_sources(keys, lev, how, rng))
+    n = rng.lognormal(0.0, 2.0, size=(keys.shape[0], S)).astype(np.float32 if dens == "f32" else np.float64)
+    tree, d = rt.Octree(_dev(keys), _dev(lev)), _dev(n)
+    cut = keys.shape[0] // 16 - 32
+    tree.reset_stats()
+    want = torch.cat([rt.trace_columns(tree, s, nside, d, mode) for s in src.split(cut)])
+    want_st = _stats(tree)
+    for again in range(2):  # the second call finds the first one's tables
+        tree.reset_stats()
+        got = rt.trace_columns(tree, src, nside, d, mode)
+        assert _stats(tree) == want_st
+        assert torch.equal(got, want), float((got - want).abs().max())
+    # another offset on the same handle, then the first again
+    moved = src + 2.0 ** -20
+    w2 = torch.cat([rt.trace_columns(tree, s, nside, d, mode) for s in moved.split(cut)])
+    assert torch.equal(rt.trace_columns(tree, moved, nside, d, mode), w2)
+    assert torch.equal(rt.trace_columns(tree, src, nside, d, mode), want)
+    # epilogues: nd terms per source in another order, each within 2^-53 of the
+    # sum of non-negative terms; A_V,eff takes a logarithm of it
+    for kind in ("av_eff", "beta", "attenuation"):
+        e = rt.trace_epilogue(tree, src, nside, d, kind, [1.0] * S, 0.05, mode=mode)
+        r = torch.cat([rt.trace_epilogue(tree, s, nside, d, kind, [1.0] * S, 0.05, mode=mode) for s in src.split(cut)])
+        torch.testing.assert_close(e, r, rtol=1e-13, atol=1e-13)
+    tree.close()
+
+
+def test_captured_call_walks(rt):
+    """Under stream capture the call takes the walk (its scratch could move
+    before a replay) and replays to the same columns."""
+    import torch
+    keys, lev = uniform_octree(5)
+    src = _dev(_sources(keys, lev, "centres", None))
+    d = torch.rand((keys.shape[0], 4), device="cuda")
+    tree = rt.Octree(_dev(keys), _dev(lev))
+    want = rt.trace_columns(tree, src, 1, d)
+    out = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        rt.trace_columns(tree, src, 1, d, out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    tree.close()
