@@ -122,19 +122,19 @@ __device__ __forceinline__ long long lookup_leaf(const DevTree& t, uint32_t cx, 
     const uint64_t M = interleave3(cx, cy, cz);
     const int csh = 3 * (kDepth - t.T);
     const uint64_t cell = M >> csh;
-    const uint64_t e = __ldg(t.table + cell);
-    const int code = (int)(e & 63u);
-    long long j = (long long)(e >> 6);
-    if (code <= kDepth) {
-        if (code > t.T) {
-            const uint64_t local = (M & ((1ull << csh) - 1ull)) >> (3 * (kDepth - code));
+    const uint2 e = __ldg((const uint2*)t.table + cell);
+    const uint32_t code = e.y;
+    long long j = (long long)e.x;
+    if (code < kCellMixed) {
+        if (code >= kCellLeaves) {
+            const uint64_t local = (M & ((1ull << csh) - 1ull)) >> (3 * (int)(code - kCellLeaves));
             j += (long long)local;
         }
-    } else if (code == kCodeHole) {
+    } else if (code == kCellHole) {
         return -1;
     } else {
         const uint64_t ncell = 1ull << (3 * t.T);
-        long long hi = (cell + 1 < ncell) ? (long long)(__ldg(t.table + cell + 1) >> 6) : t.n;
+        long long hi = (cell + 1 < ncell) ? (long long)__ldg((const uint2*)t.table + cell + 1).x : t.n;
         long long lo = j;  // keys[lo] == cell base <= M
         while (hi - lo > 1) {
             const long long mid = (lo + hi) >> 1;
@@ -1018,215 +1018,358 @@ __device__ __forceinline__ int floor_small(float v)
     return __float_as_int(__fadd_rd(v, 12582912.0f)) - 0x4B400000;
 }
 
-// Leaf containing the depth-21 point c, and its level.  The coarse table gives
-// the leaf directly for a coarse cell inside one leaf or of one level (no key
-// or level is read then); a mixed cell is searched by key.  -1: no leaf.
-__device__ __forceinline__ long long find_leaf(const DevTree& t, const uint32_t c[3], int& level)
+// The rarer kinds of coarse cell, out of line (the octree by value: a reference
+// would put the caller's into local memory): leaves two or more levels below the table, and a mixed cell, searched
+// by key.  Leaf in the low half, log2 of its size in the high one; all ones: no
+// leaf.
+static __device__ __noinline__ uint64_t find_in_cell(const DevTree t, uint32_t x, uint32_t y, uint32_t z, uint32_t cell,
+                                              uint32_t first, uint32_t code)
 {
-    const int s = kDepth - t.T;
-    const uint32_t cell = (s_spread10[(c[0] >> s) & 1023u] | (s_spread10[(c[1] >> s) & 1023u] << 1) |
-                           (s_spread10[(c[2] >> s) & 1023u] << 2)) &
-                          ((1u << (3 * t.T)) - 1u);
-    const uint64_t e = __ldg(t.table + cell);
-    const int code = (int)(e & 63u);
-    const long long first = (long long)(e >> 6);
-    if (code <= t.T) {
-        level = code;
-        return first;
+    if (code < kCellMixed) {
+        const int ls = (int)(code - kCellLeaves);
+        const uint32_t mask = (1u << (kDepth - t.T - ls)) - 1u;  // the bits of the index within the cell
+        return table_entry((uint32_t)(first + (uint32_t)interleave3((x >> ls) & mask, (y >> ls) & mask, (z >> ls) & mask)),
+                           (uint32_t)ls);
     }
-    if (code <= kDepth) {
-        const int sl = kDepth - code, nb = code - t.T;  // nb: bits per axis of the index within the cell
-        const uint32_t mask = (1u << nb) - 1u;
-        level = code;
-        if (nb == 1)  // one level below the table: the octant
-            return first + (long long)(((c[0] >> sl) & 1u) | (((c[1] >> sl) & 1u) << 1) | (((c[2] >> sl) & 1u) << 2));
-        if (nb <= 10)  // the 30-bit interleave suffices
-            return first + (long long)((s_spread10[(c[0] >> sl) & mask] | (s_spread10[(c[1] >> sl) & mask] << 1) |
-                                        (s_spread10[(c[2] >> sl) & mask] << 2)) &
-                                       ((1u << (3 * nb)) - 1u));
-        const uint64_t local = spread21((c[0] >> sl) & mask) | (spread21((c[1] >> sl) & mask) << 1) |
-                               (spread21((c[2] >> sl) & mask) << 2);
-        return first + (long long)local;
-    }
-    if (code == kCodeHole) return -1;
-    const uint64_t M = interleave3(c[0], c[1], c[2]);
-    const uint64_t ncell = 1ull << (3 * t.T);
-    long long hi = ((uint64_t)cell + 1 < ncell) ? (long long)(__ldg(t.table + cell + 1) >> 6) : t.n;
-    long long lo = first;  // keys[lo] == cell base <= M
+    if (code == kCellHole) return ~0ull;
+    const uint64_t M = interleave3(x, y, z);
+    const uint32_t ncell = 1u << (3 * t.T);
+    long long hi = cell + 1 < ncell ? (long long)__ldg((const uint2*)t.table + cell + 1).x : t.n;
+    long long lo = (long long)first;  // keys[lo] == cell base <= M
     while (hi - lo > 1) {
         const long long mid = (lo + hi) >> 1;
         if (__ldg(t.keys + mid) <= M) lo = mid;
         else hi = mid;
     }
     const uint64_t key = __ldg(t.keys + lo);
-    level = __ldg(t.levels + lo);
-    if (M - key >= (1ull << (3 * (kDepth - level)))) return -1;
-    return lo;
+    const uint32_t ls = kDepth - __ldg(t.levels + lo);
+    return M - key < (1ull << (3 * ls)) ? table_entry((uint64_t)lo, ls) : ~0ull;
+}
+
+// Leaf containing the depth-21 point c and log2 of its size.  The coarse table
+// gives the leaf directly for a coarse cell inside one leaf or of one level (no
+// key or level is read then).  False: no leaf.
+__device__ __forceinline__ bool find_leaf(const DevTree& t, const uint32_t c[3], uint32_t& j, uint32_t& ls)
+{
+    const int s = kDepth - t.T;
+    const uint32_t tmask = (1u << t.T) - 1u;  // T <= 10: inside the spread table
+    const uint32_t cell = s_spread10[(c[0] >> s) & tmask] + 2u * s_spread10[(c[1] >> s) & tmask] +
+                          4u * s_spread10[(c[2] >> s) & tmask];
+    const uint2 e = __ldg((const uint2*)t.table + cell);
+    j = e.x;
+    ls = e.y;
+    if (e.y < kCellLeaves) return true;
+    ls = e.y - kCellLeaves;
+    if ((int)ls + 1 == s) {  // one level below the table: the octant
+        j += ((c[0] >> ls) & 1u) + 2u * ((c[1] >> ls) & 1u) + 4u * ((c[2] >> ls) & 1u);
+        return true;
+    }
+    const uint64_t found = find_in_cell(t, c[0], c[1], c[2], cell, e.x, e.y);
+    j = (uint32_t)found;
+    ls = (uint32_t)(found >> 32) & 31u;
+    return found != ~0ull;
+}
+
+// Exit set of a step whose two smallest times are within the certified margin,
+// out of line: bits 0-2 the exit axes, bit 3 set if FP64 decided.
+template <int VM, bool QZ>
+__device__ __noinline__ unsigned near_exit(const DevTree t, const DirConst* __restrict__ dp,
+                                           const double* __restrict__ src, float A0, float A1, float A2, float t0,
+                                           float t1, float t2, float cE)
+{
+    const float Af[3] = {A0, A1, A2};
+    float th[3] = {t0, t1, t2}, ih[3], a[3], z[3];
+    int qi[3], bs;
+    uint32_t qf[3];
+    source_fixed(src, t, qi, qf, a, z);
+#pragma unroll
+    for (int b = 0; b < 3; b++) ih[b] = (VM & (1 << b)) ? fabsf(__ldg(&dp->ih[b])) * 0x1p-21f : 0.f;
+    WalkCounters wc = {0u, 0u, 0u};
+    const unsigned E = exit_set<VM, QZ, true>(th, Af, qf, ih, __ldg(&dp->flags), cE, dp, bs, wc);
+    return E | (wc.exit_fb << 3);
+}
+
+// Point behind the exit face, on a finer neighbour's own lattice, where the
+// common step's position is too near one of the neighbour's faces: on the axes
+// that move and are not in E the lower end of the certified FP32 interval of
+// the exit point, clamped into the leaf left (lower corner lo, size), or, where
+// the leaf there does not hold the whole interval, the FP64 position of the
+// definition, floor((Q + t_out m) 2^21).  Unreflected; x on the other axes.
+// Packed 21 bits an axis, bit 63 set if FP64 decided.  the, A: exit time (box
+// lengths) and mirrored far-face distance of the lowest axis of E.
+template <int VM, bool QZ>
+__device__ __noinline__ uint64_t near_point(const DevTree t, const DirConst* __restrict__ dp,
+                                            const double* __restrict__ src, unsigned E, float the, float A, uint32_t x0,
+                                            uint32_t x1, uint32_t x2, uint32_t lo0, uint32_t lo1, uint32_t lo2, uint32_t size)
+{
+    uint32_t x[3] = {x0, x1, x2}, chi[3] = {x0, x1, x2};
+    const uint32_t lo[3] = {lo0, lo1, lo2};
+    int qi[3];
+    uint32_t qf[3];
+    float ph[3], pl[3];
+    source_fixed(src, t, qi, qf, ph, pl);
+    const int bs = __ffs(E) - 1;
+    const float ihe = __ldg(&dp->ih[bs]);
+    bool wide = false;
+#pragma unroll
+    for (int b = 0; b < 3; b++) {
+        if ((VM & (1 << b)) && !(E & (1u << b))) {
+            const int hib = (int)(lo[b] + size - 1u);
+            const float m32 = __ldg(&dp->m32[b]);
+            const float mw = __fmul_rn(the * 0x1p21f, m32);  // depth-21 units
+            const float w = QZ ? mw : __fadd_rn(mw, ph[b]);
+            const float del = (fabsf(mw) + fabsf(w)) * 0x1p-21f + fabsf(m32) * fabsf(ihe) * 0x1p-22f + 0x1p-22f;
+            // |w| + del < 2^22: floor by adding 1.5 * 2^23 rounded down
+            const int l0 = qi[b] + floor_small(__fsub_rd(w, del));
+            const int l1 = qi[b] + floor_small(__fadd_ru(w, del));
+            x[b] = (uint32_t)min(max(l0, (int)lo[b]), hib);
+            chi[b] = (uint32_t)min(max(l1, (int)lo[b]), hib);
+            wide |= chi[b] != x[b];
+        }
+    }
+    uint64_t fb = 0;
+    if (wide) {
+        uint32_t j, ls;
+        bool fp64 = !find_leaf(t, x, j, ls);
+#pragma unroll
+        for (int b = 0; b < 3; b++) fp64 |= chi[b] >= (x[b] & ~((1u << ls) - 1u)) + (1u << ls);
+        if (fp64) {
+            fb = 1ull << 63;
+            const long long De = face_distance<true>(A, sel3(qf, bs), __ldg(&dp->flags), bs);
+            const double te = __dmul_rn(__dmul_rn(__ll2double_rn(De), 0x1p-53), fabs(__ldg(&dp->inv[bs])));
+#pragma unroll
+            for (int b = 0; b < 3; b++) {
+                if ((VM & (1 << b)) && !(E & (1u << b))) {
+                    const long long qb = ((long long)qi[b] << 32) | (long long)qf[b];
+                    const double Qb = __dmul_rn(__ll2double_rn(qb), 0x1p-53);
+                    const double P = __dadd_rn(Qb, __dmul_rn(te, __ldg(&dp->m[b])));
+                    double f = floor(__dmul_rn(P, 0x1p21));
+                    f = fmax(f, (double)lo[b]);
+                    f = fmin(f, (double)(lo[b] + size - 1u));
+                    x[b] = (uint32_t)f;
+                }
+            }
+        }
+    }
+    return (uint64_t)x[0] | (uint64_t)x[1] << 21 | (uint64_t)x[2] << 42 | fb;
+}
+
+// find_leaf out of line, for the step after near_point.
+static __device__ __noinline__ uint64_t find_leaf_packed(const DevTree t, uint64_t p)
+{
+    const uint32_t x[3] = {(uint32_t)p & 0x1fffffu, (uint32_t)(p >> 21) & 0x1fffffu, (uint32_t)(p >> 42) & 0x1fffffu};
+    uint32_t j, ls;
+    return find_leaf(t, x, j, ls) ? table_entry(j, ls) : ~0ull;
 }
 
 // Walk of one ray through a general octree, F32-Kahan arithmetic, moving axes
-// VM (compile time).  Exit decisions as in walk_f32k_grid.  The next leaf is
-// looked up at the lower corner of the current leaf on the non-stepped axes;
-// only when that neighbour is finer, at the FP32 position of the non-stepped
-// axes when its certified interval lies inside the leaf found, else at the
-// FP64 position.
+// VM (compile time), in the mirrored frame of walk_f32k_grid: a moving axis
+// with m_b < 0 is reflected (cell c -> 2^21 - 1 - c = c ^ (2^21 - 1), and a
+// source integer qi -> 2^21 - qi), so that every exit face is the upper one,
+// at hi_b, every distance, reciprocal and time is positive, and a step needs
+// no sign.  Points are reflected back (one XOR) where a leaf is looked up.
+//
+// One exit axis ahead of the others by the certified margin is the common
+// step: it takes the smallest and the second smallest time (five minima and
+// maxima) and compares; anything nearer goes through exit_set.
+//
+// The next leaf is looked up at the FP32 position of the exit point on the
+// non-stepped axes, clamped into the current leaf.  A leaf at least as large as
+// the current one covers the whole face-adjacent cell of the current size
+// (octree cells are aligned), so any position on the face finds it.  A finer one
+// is the leaf of the definition if it holds the position with kNearPoint lattice
+// cells to spare on each side, more than the position's error; else (one step
+// in a thousand at leaves of 4096 lattice cells) near_point decides.
+//
+// Bound: instruction issue.
 template <int VM, bool QZ, class V, class R = NoResume>
 __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* __restrict__ dp,
                                               const double* __restrict__ src, long long cap, V& vis,
                                               WalkCounters& wc, R* rs = nullptr)
 {
-    // The direction's constants (ih, il, m32) are read from the direction
-    // table where they are used: one broadcast load per warp, kept out of the
-    // per-ray registers.
-    const int flags = __ldg(&dp->flags);
-    float ph[3], pl[3], qif[3];  // qif: 2^23 + qi, exact
-    int qi[3];
-    uint32_t qf[3], c[3];
+    constexpr int nvm = ((VM >> 0) & 1) + ((VM >> 1) & 1) + ((VM >> 2) & 1);
+    constexpr uint32_t kOnes = (1u << kDepth) - 1u;
+    const float inf = __int_as_float(0x7f800000);
+    const bool full = ((t.ext[0] & t.ext[1] & t.ext[2]) >> kDepth) != 0u;  // the whole cube
+    // qif: 2^23 + mirrored source integer, exact; ihs: the reciprocal, negative
+    // on a reflected axis, scaled by 2^-21 (exact), so that times are in box
+    // lengths
+    float ph[3], pl[3], qif[3], ihs[3];
+    uint32_t hi[3], c[3];  // c: mirrored point
     float cE = 0.f;
-    const int st = source_fixed(src, t, qi, qf, ph, pl);
-    if (st != RT_OK) return st;
+    // all ones on a reflected axis
+    auto mir = [&](int b) { return (uint32_t)(__float_as_int(ihs[b]) >> 31); };
+    constexpr int kNearPoint = 8;  // (|mw| + |w|) 2^-21 <= 2, |m| |ihe| 2^-22 <= 1 below the test's |ihe|, 2^-22, a floor
+    auto lower = [&](int b, uint32_t sz) { return mir(b) ? (1u << kDepth) - hi[b] : hi[b] - sz; };  // unreflected
+    {
+        int qi[3];
+        uint32_t qf[3];
+        const int st = source_fixed(src, t, qi, qf, ph, pl);
+        if (st != RT_OK) return st;
 #pragma unroll
-    for (int b = 0; b < 3; b++) {
-        qif[b] = __int_as_float(0x4B000000 | qi[b]);
-        c[b] = (uint32_t)qi[b];
-        if (VM & (1 << b)) cE = fmaxf(cE, fabsf(dir_const(&dp->ih[b])) * kEA);
+        for (int b = 0; b < 3; b++) {
+            ihs[b] = (VM & (1 << b)) ? __ldg(&dp->ih[b]) * 0x1p-21f : 0.f;
+            const bool neg = mir(b) != 0u;
+            c[b] = ((uint32_t)qi[b] ^ mir(b)) & kOnes;
+            qif[b] = __int_as_float(0x4B000000 | (neg ? (1 << kDepth) - qi[b] : qi[b]));
+            if (neg) {
+                ph[b] = -ph[b];
+                pl[b] = -pl[b];
+            }
+            if (QZ) ph[b] = pl[b] = 0.f;
+            if (VM & (1 << b)) cE = fmaxf(cE, fabsf(ihs[b]) * kEA);
+        }
     }
-    int level;
-    long long j;
-    uint32_t size, lo[3];
+    uint32_t j, size;
     float tih = 0.f, til = 0.f;
     if (R::enabled && rs->s->status == 1) {
         j = rs->s->j;
-        level = rs->s->level;
-        size = 1u << (kDepth - level);
+        size = 1u << (kDepth - rs->s->level);
 #pragma unroll
-        for (int b = 0; b < 3; b++) lo[b] = rs->s->lo[b];
+        for (int b = 0; b < 3; b++) hi[b] = mir(b) ? (1u << kDepth) - rs->s->lo[b] : rs->s->lo[b] + size;
         tih = rs->s->th;
         til = rs->s->tl;
     } else {
-        j = find_leaf(t, c, level);
-        if (j < 0) return RT_ERR_LOOKUP_MISS;
-        size = 1u << (kDepth - level);
+        uint32_t x[3], ls;
 #pragma unroll
-        for (int b = 0; b < 3; b++) lo[b] = c[b] & ~(size - 1u);
+        for (int b = 0; b < 3; b++) x[b] = (c[b] ^ mir(b)) & kOnes;
+        if (!find_leaf(t, x, j, ls)) return RT_ERR_LOOKUP_MISS;
+        size = 1u << ls;
+#pragma unroll
+        for (int b = 0; b < 3; b++) hi[b] = (c[b] | (size - 1u)) + 1u;
     }
     // cap >= 1; a resumed walk counts from the ray's start (wc.nseg holds it)
     const uint32_t lim = (R::enabled ? 0u : wc.nseg) + (uint32_t)min(cap, (long long)0x7fffffff);
     for (;;) {
-        if (R::enabled && !rs->inside(j)) {
-            rs->s->j = (uint32_t)j;
+        if (R::enabled && !rs->inside((long long)j)) {
+            rs->s->j = j;
 #pragma unroll
-            for (int b = 0; b < 3; b++) rs->s->lo[b] = lo[b];
+            for (int b = 0; b < 3; b++) rs->s->lo[b] = lower(b, size);
             rs->s->level = (uint8_t)(kDepth - (31 - __clz(size)));
             rs->s->th = tih;
             rs->s->tl = til;
             rs->s->nseg = wc.nseg;
             return kSuspended;
         }
-        vis.pre((uint32_t)j);
-        float Af[3], th[3], tl[3], ih[3];
+        vis.pre(j);
+        float Af[3], sd[3], th[3];
 #pragma unroll
         for (int b = 0; b < 3; b++) {
-            Af[b] = th[b] = tl[b] = ih[b] = 0.f;
+            Af[b] = sd[b] = 0.f;
+            th[b] = inf;
             if (VM & (1 << b)) {
-                ih[b] = dir_const(&dp->ih[b]);
-                const uint32_t F = ((flags >> (3 + b)) & 1) ? lo[b] + size : lo[b];
                 // (2^23 + F) - (2^23 + qi) = F - qi: integers below 2^24, exact
-                Af[b] = __fsub_rn(__int_as_float(0x4B000000 | (int)F), qif[b]);
-                if (QZ) {
-                    th[b] = __fmul_rn(Af[b], ih[b]);
-                } else {
-                    th[b] = __fmul_rn(__fsub_rn(Af[b], ph[b]), ih[b]);
-                }
+                Af[b] = __fsub_rn(__int_as_float(0x4B000000 | (int)hi[b]), qif[b]);
+                sd[b] = QZ ? Af[b] : __fsub_rn(Af[b], ph[b]);
+                th[b] = __fmul_rn(sd[b], fabsf(ihs[b]));
             }
         }
-        int bs;
-        const unsigned E = exit_set<VM, QZ, false>(th, Af, qf, ih, flags, cE, dp, bs, wc);
+        const float m01 = fminf(th[0], th[1]);
+        const float t1 = fminf(m01, th[2]);
+        bool e[3];
+#pragma unroll
+        for (int b = 0; b < 3; b++) e[b] = (VM & (1 << b)) && th[b] == t1;
+        if (nvm > 1) {
+            const float t2 = fminf(fmaxf(th[0], th[1]), fmaxf(m01, th[2]));
+            bool near = !(__fsub_rn(t2, t1) > (t2 + t1) * kER + 2.f * cE);
+            if (QZ && near && t2 == t1) {
+                // two axes of equal reciprocal and distance tie exactly, the
+                // third beyond the margin: e holds the two
+                const int flags = __ldg(&dp->flags);
+                const float t3 = fmaxf(fmaxf(th[0], th[1]), th[2]);
+                const bool tie = (e[0] && e[1] && inv_equal(flags, 0, 1) && Af[0] == Af[1]) ||
+                                 (e[0] && e[2] && inv_equal(flags, 0, 2) && Af[0] == Af[2]) ||
+                                 (e[1] && e[2] && inv_equal(flags, 1, 2) && Af[1] == Af[2]);
+                near = !(tie && (nvm < 3 || __fsub_rn(t3, t1) > (t3 + t1) * kER + 2.f * cE));
+            }
+            if (near) {
+                const unsigned E = near_exit<VM, QZ>(t, dp, src, Af[0], Af[1], Af[2], th[0], th[1], th[2], cE);
+                wc.exit_fb += E >> 3;
+#pragma unroll
+                for (int b = 0; b < 3; b++) e[b] = (E >> b) & 1u;
+            }
+        }
+        // the lowest exit axis: its time in double-float.  s = fl(A - ph) with
+        // A an integer, 0 or at least |ph|: (A - s) - ph is the rounding error
+        const float Ae = e[0] ? Af[0] : (e[1] ? Af[1] : Af[2]);
+        const float ihe = e[0] ? ihs[0] : (e[1] ? ihs[1] : ihs[2]);
+        const float* ilp = e[0] ? &dp->il[0] : (e[1] ? &dp->il[1] : &dp->il[2]);
+        const float ila = __ldg(ilp) * 0x1p-21f;
+        const float ile = __int_as_float(__float_as_int(ila) ^ (__float_as_int(ihe) & (int)0x80000000));
         float the, tle;
-        exit_time<QZ>(sel3(Af, bs), sel3(ph, bs), sel3(pl, bs), sel3(ih, bs), dir_const(&dp->il[bs]), the, tle);
-        const float ds = __fmul_rn(__fadd_rn(__fsub_rn(the, tih), __fsub_rn(tle, til)), 0x1p-21f);
+        if (QZ) {
+            the = __fmul_rn(Ae, fabsf(ihe));
+            tle = __fmaf_rn(Ae, ile, __fmaf_rn(Ae, fabsf(ihe), -the));
+        } else {
+            const float se = e[0] ? sd[0] : (e[1] ? sd[1] : sd[2]);
+            const float pe = e[0] ? ph[0] : (e[1] ? ph[1] : ph[2]);
+            const float le = e[0] ? pl[0] : (e[1] ? pl[1] : pl[2]);
+            const float rl = __fsub_rn(__fsub_rn(__fsub_rn(Ae, se), pe), le);
+            the = __fmul_rn(se, fabsf(ihe));
+            tle = __fadd_rn(__fmaf_rn(se, fabsf(ihe), -the), __fmaf_rn(se, ile, __fmul_rn(rl, fabsf(ihe))));
+        }
+        const float ds = __fadd_rn(__fsub_rn(the, tih), __fsub_rn(tle, til));
         tih = the;
         til = tle;
         vis.acc(ds);
         wc.nseg++;
-        // Step the exit axes; a moving axis that does not step first takes the
-        // leaf's lower corner.  The leaf found there is the neighbour of the
-        // definition unless it is finer than the current leaf: a leaf at least
-        // as large covers the whole face-adjacent cell of the current size
-        // (octree cells are aligned), so any exit point on the face lands in it.
-        bool leaving = false;
+        // the exit axes enter the next cell, the others take the exit point; a
+        // fixed coordinate stays inside every leaf on the path
+        const float t21 = the * 0x1p21f;  // depth-21 units
+        uint32_t out = 0u;
 #pragma unroll
         for (int b = 0; b < 3; b++) {
-            const int pos = (flags >> (3 + b)) & 1;
-            if ((VM & (1 << b)) && (E & (1u << b))) {
-                if (pos ? (lo[b] + size >= t.ext[b]) : (lo[b] == 0)) leaving = true;
-                c[b] = pos ? lo[b] + size : lo[b] - 1;
-            } else if (!(VM & (1 << b))) {
-                c[b] = (uint32_t)qi[b];  // a fixed coordinate stays inside every leaf on the path
-            } else {
-                c[b] = lo[b];
+            if (VM & (1 << b)) {
+                const float mw = __fmul_rn(t21, fabsf(dir_const(&dp->m32[b])));
+                const float w = QZ ? mw : __fadd_rn(mw, ph[b]);
+                // floor(w) by adding 1.5 * 2^23 rounded down, plus the source integer
+                const int p = __float_as_int(__fadd_rd(w, 12582912.0f)) + (__float_as_int(qif[b]) - 0x4B400000 - 0x4B000000);
+                c[b] = e[b] ? hi[b] : (uint32_t)min(max(p, (int)(hi[b] - size)), (int)hi[b] - 1);
+                out |= c[b];
             }
+        }
+        bool leaving = (out >> kDepth) != 0u;  // past the cube's upper face
+        if (!full) {
+#pragma unroll
+            for (int b = 0; b < 3; b++) leaving |= (VM & (1 << b)) && e[b] && !mir(b) && hi[b] >= t.ext[b];
         }
         if (leaving) break;
+        uint32_t x[3], ls;
+#pragma unroll
+        for (int b = 0; b < 3; b++) x[b] = (c[b] ^ mir(b)) & kOnes;
         const uint32_t size0 = size;  // the current leaf's size
-        j = find_leaf(t, c, level);
-        size = 1u << (kDepth - level);
-        if ((VM & ~E) != 0u && j >= 0 && size < size0) {
-            // a finer neighbour: position the moving non-exit axes on a
-            // certified interval around the exit point
-            const float ihe = sel3(ih, bs);
-            bool wide = false;
-            uint32_t chi[3];
+        bool hit = find_leaf(t, x, j, ls);
+        size = 1u << ls;
+        if (nvm > 1 && size < size0) {
+            uint32_t apart = fabsf(ihe) < 2.f ? 0u : ~0u;
 #pragma unroll
             for (int b = 0; b < 3; b++) {
-                chi[b] = c[b];
-                if ((VM & (1 << b)) && !(E & (1u << b))) {
-                    const uint32_t hib = lo[b] + size0 - 1;
-                    const float m32 = dir_const(&dp->m32[b]);
-                    const float mw = __fmul_rn(the, m32);
-                    const float w = QZ ? mw : __fadd_rn(mw, ph[b]);
-                    const float del = (fabsf(mw) + fabsf(w)) * 0x1p-21f + fabsf(m32) * fabsf(ihe) * 0x1p-22f +
-                                      0x1p-22f;
-                    // |w| + del < 2^22: floor by adding 1.5 * 2^23 rounded down
-                    const int l0 = qi[b] + floor_small(__fsub_rd(w, del));
-                    const int l1 = qi[b] + floor_small(__fadd_ru(w, del));
-                    c[b] = (uint32_t)min(max(l0, (int)lo[b]), (int)hib);
-                    chi[b] = (uint32_t)min(max(l1, (int)lo[b]), (int)hib);
-                    wide |= chi[b] != c[b];
+                if ((VM & (1 << b)) && !e[b]) {
+                    const int a = max((int)c[b] - kNearPoint, (int)(hi[b] - size0));
+                    const int z = min((int)c[b] + kNearPoint, (int)hi[b] - 1);
+                    apart |= (uint32_t)(a ^ z);
                 }
             }
-            j = find_leaf(t, c, level);
-            size = 1u << (kDepth - level);
-            if (wide && j >= 0) {
+            if (!hit || (apart & ~(size - 1u)) != 0u) {
+                const unsigned E = (e[0] ? 1u : 0u) | (e[1] ? 2u : 0u) | (e[2] ? 4u : 0u);
 #pragma unroll
-                for (int b = 0; b < 3; b++)
-                    if (chi[b] >= (c[b] & ~(size - 1u)) + size) j = -2;
-            }
-            if (j == -2 || (j < 0 && wide)) {
-                // FP64 position of the definition: floor((Q + t_out m) 2^21)
-                wc.lookup_fb++;
-                const long long De = ((long long)small_float_to_int(sel3(Af, bs)) << 32) - (long long)sel3(qf, bs);
-                const double te = __dmul_rn(__dmul_rn(__ll2double_rn(De), 0x1p-53), __ldg(&dp->inv[bs]));
+                for (int b = 0; b < 3; b++) x[b] = (c[b] ^ mir(b)) & kOnes;
+                const uint64_t p = near_point<VM, QZ>(t, dp, src, E, the, Ae, x[0], x[1], x[2], lower(0, size0),
+                                                      lower(1, size0), lower(2, size0), size0);
+                wc.lookup_fb += (uint32_t)(p >> 63);
+                const uint64_t found = find_leaf_packed(t, p);
+                hit = found != ~0ull;
+                j = (uint32_t)found;
+                size = 1u << ((uint32_t)(found >> 32) & 31u);
 #pragma unroll
-                for (int b = 0; b < 3; b++) {
-                    if ((VM & (1 << b)) && !(E & (1u << b))) {
-                        const long long qb = ((long long)qi[b] << 32) | (long long)qf[b];
-                        const double Qb = __dmul_rn(__ll2double_rn(qb), 0x1p-53);
-                        const double P = __dadd_rn(Qb, __dmul_rn(te, __ldg(&dp->m[b])));
-                        double f = floor(__dmul_rn(P, 0x1p21));
-                        f = fmax(f, (double)lo[b]);
-                        f = fmin(f, (double)(lo[b] + size0 - 1));
-                        c[b] = (uint32_t)f;
-                    }
-                }
-                j = find_leaf(t, c, level);
-                size = 1u << (kDepth - level);
+                for (int b = 0; b < 3; b++) c[b] = ((uint32_t)(p >> (21 * b)) ^ mir(b)) & kOnes;
             }
         }
-        if (j < 0) return RT_ERR_LOOKUP_MISS;
+        if (!hit) return RT_ERR_LOOKUP_MISS;
         if (wc.nseg >= lim) return RT_ERR_STEP_LIMIT;  // the cap ends a ray that still goes on
 #pragma unroll
-        for (int b = 0; b < 3; b++) lo[b] = c[b] & ~(size - 1u);
+        for (int b = 0; b < 3; b++)
+            if (VM & (1 << b)) hi[b] = (c[b] | (size - 1u)) + 1u;
     }
     return RT_OK;
 }

@@ -12,14 +12,21 @@ constexpr int kDepth = 21;          // anchor depth of the Morton lattice
 constexpr int kMaxSpecies = 8;
 constexpr int kBaseTableLevel = 7;  // coarse table level for every tree (8^7 = 2M entries at most)
 constexpr int kMaxTableLevel = 10;  // deepest coarse table (the lookup's cell index holds 30 bits)
-constexpr int kCodeHole = 62;       // coarse cell outside the domain box
-constexpr int kCodeMixed = 63;      // coarse cell with leaves of several levels
+// Coarse-table entries: the first leaf in the low half, in the high half what
+// is there: log2 of the leaf's size for a cell inside one leaf, kCellLeaves
+// more than that for a cell whose leaves all have one finer level, or one of
+// the two codes after it.  Whole halves, so that a lookup takes neither without
+// a 64-bit shift.
+constexpr uint32_t kCellLeaves = 32;
+constexpr uint32_t kCellMixed = 64;  // leaves of several levels
+constexpr uint32_t kCellHole = 65;   // outside the domain box
+constexpr uint64_t table_entry(uint64_t first, uint32_t code) { return first | (uint64_t)code << 32; }
 
 // Device view of an octree handle.
 struct DevTree {
     const uint64_t* keys;
     const uint8_t* levels;
-    const uint64_t* table;   // [8^T] entries: (first leaf << 6) | code
+    const uint64_t* table;   // [8^T] entries (table_entry)
     int64_t n;
     uint32_t ext[3];
     int T;                   // coarse table level

@@ -39,8 +39,15 @@ static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
 static DirConst g_dirs_stage[4][kNoAllocMaxDirs];
 static bool g_dirs_ready[4];
 static double g_dirs_host[3 * kNoAllocMaxDirs];
-static const uint64_t kRootEntries[23] = {0,  1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11,
-                                          12, 13, 14, 15, 16, 17, 18, 19, 20, 21, (uint64_t)kCodeMixed};
+struct RootEntries {
+    uint64_t e[23];
+    constexpr RootEntries() : e()
+    {
+        for (int l = 0; l <= kDepth; l++) e[l] = table_entry(0, (l ? kCellLeaves : 0u) + (uint32_t)(kDepth - l));
+        e[22] = table_entry(0, kCellMixed);
+    }
+};
+static constexpr RootEntries kRootEntries;
 static std::mutex g_noalloc_mu;
 static NoAllocScratch* g_noalloc_ptr[64];  // device address of the array, per device
 
@@ -143,7 +150,7 @@ extern "C" int rt_trace_columns_noalloc(const uint64_t* d_keys, const uint8_t* d
     // cube, else a key search over all leaves) and the directions, copied from
     // host data that never changes once computed
     if (cudaMemsetAsync(&sc->stats, 0, sizeof(DevStats), s) != cudaSuccess ||
-        cudaMemcpyAsync(&sc->root_entry, &kRootEntries[uniform ? max_level : 22], sizeof(uint64_t),
+        cudaMemcpyAsync(&sc->root_entry, &kRootEntries.e[uniform ? max_level : 22], sizeof(uint64_t),
                         cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(sc->dirs, staged_directions(nside), sizeof(DirConst) * nd, cudaMemcpyHostToDevice,
                         s) != cudaSuccess)

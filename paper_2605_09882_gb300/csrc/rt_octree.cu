@@ -93,10 +93,11 @@ __device__ __forceinline__ int64_t lower_bound_keys(const uint64_t* keys, int64_
 }
 
 // One entry per coarse cell C (Morton index at level T):
-//   code l <= T : the cell lies in leaf `first` (level l);
-//   code l > T  : every leaf in the cell has level l, leaf = first + local index;
-//   kCodeMixed  : binary search in [first, next cell's first);
-//   kCodeHole   : the cell starts outside the domain box.
+//   21 - l               : the cell lies in leaf `first` (level l <= T);
+//   kCellLeaves + 21 - l : every leaf in the cell has level l > T, leaf = first +
+//                          local index;
+//   kCellMixed           : binary search in [first, next cell's first);
+//   kCellHole            : the cell starts outside the domain box.
 __global__ void k_fill_table(const uint64_t* __restrict__ keys, const uint8_t* __restrict__ levels,
                              int64_t n, int T, uint32_t ex, uint32_t ey, uint32_t ez,
                              const unsigned* lvmin, const unsigned* lvmax, uint64_t* table)
@@ -107,23 +108,23 @@ __global__ void k_fill_table(const uint64_t* __restrict__ keys, const uint8_t* _
          C += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t base = C << csh;
         const int64_t j0 = lower_bound_keys(keys, n, base);
-        int code;
+        uint32_t code;
         int64_t first = j0;
         if (compact21(base) >= ex || compact21(base >> 1) >= ey || compact21(base >> 2) >= ez) {
-            code = kCodeHole;
+            code = kCellHole;
         } else if (j0 > 0 && keys[j0 - 1] + (1ull << (3 * (kDepth - levels[j0 - 1]))) > base) {
-            code = levels[j0 - 1];
+            code = kDepth - levels[j0 - 1];
             first = j0 - 1;
         } else if (j0 < n && keys[j0] == base && (int)levels[j0] <= T) {
-            code = levels[j0];
+            code = kDepth - levels[j0];
         } else if (lvmin[C] == lvmax[C]) {
             const int l = (int)lvmin[C];
             const int64_t j1 = lower_bound_keys(keys, n, base + (1ull << csh));
-            code = (j1 - j0 == (int64_t)(1ull << (3 * (l - T)))) ? l : kCodeMixed;
+            code = (j1 - j0 == (int64_t)(1ull << (3 * (l - T)))) ? kCellLeaves + kDepth - l : kCellMixed;
         } else {
-            code = kCodeMixed;
+            code = kCellMixed;
         }
-        table[C] = ((uint64_t)first << 6) | (uint64_t)code;
+        table[C] = table_entry((uint64_t)first, code);
     }
 }
 
