@@ -126,6 +126,23 @@ const DirConst* direction_table(int dev, int nside, int* status) { return dir_ta
 
 int sm_count_of(int dev) { return sm_count(dev); }
 
+// With fewer groups than the launch has warps, a pop takes one group, and with
+// fewer rays than lanes a warp takes fewer rays: each ray is a serial chain of
+// lookups whose latency nothing hides when the machine is not full, and a
+// warp's lanes wait for one another's at every divergent branch.  (Direction
+// groups need whole warps.)
+#ifndef RT_MIN_GW
+#define RT_MIN_GW 8
+#endif
+void spread_rays(TraceArgs& a, long long warps)
+{
+    const long long rays = (long long)(a.layout ? a.n_src : a.n_src_pad) * a.nd;
+    a.batch = (int)std::max<long long>(1, std::min<long long>(a.batch, rays / 32 / std::max<long long>(1, warps)));
+    a.gw = 32;
+    if (a.dgroup <= 1 && !a.pair)
+        while (a.gw > RT_MIN_GW && rays / a.gw < warps) a.gw >>= 1;
+}
+
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Common argument handling of the trace entry points.
@@ -166,6 +183,7 @@ int prepare_trace(const rt_octree* t, const double* d_src, int64_t n_src, int ns
     a.S = S;
     a.st = t->st;
     a.batch = g_batch;
+    a.gw = 32;
     a.layout = ray_layout(n_src);
     a.dgroup = 1;
     return RT_OK;
@@ -309,7 +327,9 @@ int rt::trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_sr
                            : occupancy_fwd(0, mode, n_species, a.t.uniform_level >= 0, g_block);
     if (cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
         return cuda_error("rt_trace_columns: queue reset");
-    if (launch_forward(a, mode, g_block, grid_for(fit), s) != cudaSuccess)
+    const int grid = grid_for(fit);
+    spread_rays(a, (long long)grid * (g_block / 32));
+    if (launch_forward(a, mode, g_block, grid, s) != cudaSuccess)
         return cuda_error("rt_trace_columns: launch");
     return RT_OK;
 }
@@ -329,7 +349,9 @@ int rt_trace_paths(const rt_octree* t, const double* d_src, int64_t n_src, int n
     const int fit = occupancy_fwd(1, mode, 1, a.t.uniform_level >= 0, g_block);
     if (cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
         return cuda_error("rt_trace_paths: queue reset");
-    if (launch_paths(a, mode, g_block, grid_for(fit), s) != cudaSuccess)
+    const int grid = grid_for(fit);
+    spread_rays(a, (long long)grid * (g_block / 32));
+    if (launch_paths(a, mode, g_block, grid, s) != cudaSuccess)
         return cuda_error("rt_trace_paths: launch");
     return RT_OK;
 }

@@ -110,53 +110,6 @@ struct WalkCounters {
     uint32_t lookup_fb;
 };
 
-// ------------------------------------------------------------ leaf lookup
-
-// Leaf containing the depth-21 point (cx, cy, cz): coarse Morton table at
-// level T, then an O(1) index for a single-level coarse cell or a binary
-// search of the sorted keys inside a mixed one.  Returns -1 if no leaf
-// contains the point.  key/level receive the leaf's key and level.
-__device__ __forceinline__ long long lookup_leaf(const DevTree& t, uint32_t cx, uint32_t cy,
-                                                 uint32_t cz, uint64_t& key, int& level)
-{
-    const uint64_t M = interleave3(cx, cy, cz);
-    const int csh = 3 * (kDepth - t.T);
-    const uint64_t cell = M >> csh;
-    const uint2 e = __ldg((const uint2*)t.table + cell);
-    const uint32_t code = e.y;
-    long long j = (long long)e.x;
-    if (code < kCellMixed) {
-        if (code >= kCellLeaves) {
-            const uint64_t local = (M & ((1ull << csh) - 1ull)) >> (3 * (int)(code - kCellLeaves));
-            j += (long long)local;
-        }
-    } else if (code == kCellHole) {
-        return -1;
-    } else {
-        const uint64_t ncell = 1ull << (3 * t.T);
-        long long hi = (cell + 1 < ncell) ? (long long)__ldg((const uint2*)t.table + cell + 1).x : t.n;
-        long long lo = j;  // keys[lo] == cell base <= M
-        while (hi - lo > 1) {
-            const long long mid = (lo + hi) >> 1;
-            if (__ldg(t.keys + mid) <= M) lo = mid;
-            else hi = mid;
-        }
-        j = lo;
-    }
-    key = __ldg(t.keys + j);
-    level = __ldg(t.levels + j);
-    if (M - key >= (1ull << (3 * (kDepth - level)))) return -1;
-    return j;
-}
-
-__device__ __forceinline__ void leaf_box(uint64_t key, int level, uint32_t lo[3], uint32_t& size)
-{
-    lo[0] = compact21(key);
-    lo[1] = compact21(key >> 1);
-    lo[2] = compact21(key >> 2);
-    size = 1u << (kDepth - level);
-}
-
 // ---------------------------------------------------- source on the lattice
 
 // Source coordinate b truncated to the 2^-53 lattice: q = floor(x * 2^53).
@@ -222,140 +175,6 @@ struct ChunkResume {
 };
 
 // ======================================================== FP64 walk (MODE 0)
-
-// Walks one ray in FP64, the operation order of the plain definition:
-//   t_b = (F_b - Q_b) * inv_b, t_out = min_b t_b, E = {b : t_b == t_out},
-//   ds = t_out - t_in, stepped axes move to the neighbour cell, the others
-//   take floor((Q_b + t_out m_b) 2^21) clamped into the current leaf (formed
-//   only when the neighbour is finer than the current leaf; see below).
-// V::seg(j, ds) receives every segment.
-template <bool UNIFORM, class V, class R = NoResume>
-__device__ __forceinline__ int walk_fp64(const DevTree& t, const DirConst& d,
-                                         const double* __restrict__ src, long long cap, V& vis,
-                                         WalkCounters& wc, R* rs = nullptr)
-{
-    double Q[3];
-    uint32_t c[3];
-#pragma unroll
-    for (int b = 0; b < 3; b++) {
-        long long q;
-        if (!fixed_source(src[b], q)) return RT_ERR_SOURCE_OUTSIDE;
-        Q[b] = __dmul_rn(__ll2double_rn(q), 0x1p-53);
-        c[b] = (uint32_t)(q >> 32);
-        if (c[b] >= t.ext[b]) return RT_ERR_SOURCE_OUTSIDE;
-    }
-    uint32_t lo[3], size;
-    uint32_t ci[3], dil = 0;  // uniform grid: level-L cell index and its Morton index
-    long long j;
-    const int ush = kDepth - t.uniform_level;
-    if (UNIFORM) {
-#pragma unroll
-        for (int b = 0; b < 3; b++) ci[b] = c[b] >> ush;
-        dil = spread10(ci[0]) | (spread10(ci[1]) << 1) | (spread10(ci[2]) << 2);
-        j = dil;
-        size = 1u << ush;
-    } else if (R::enabled && rs->s->status == 1) {
-        j = rs->s->j;
-#pragma unroll
-        for (int b = 0; b < 3; b++) lo[b] = rs->s->lo[b];
-        size = 1u << (kDepth - rs->s->level);
-    } else {
-        uint64_t key;
-        int level;
-        j = lookup_leaf(t, c[0], c[1], c[2], key, level);
-        if (j < 0) return RT_ERR_LOOKUP_MISS;
-        leaf_box(key, level, lo, size);
-    }
-    double t_in = (R::enabled && rs->s->status == 1) ? rs->s->t : 0.0;
-    for (long long step = R::enabled ? (long long)rs->s->nseg : 0;; ++step) {
-        if (step >= cap) return RT_ERR_STEP_LIMIT;
-        if (R::enabled && !rs->inside(j)) {
-            rs->s->j = (uint32_t)j;
-#pragma unroll
-            for (int b = 0; b < 3; b++) rs->s->lo[b] = lo[b];
-            rs->s->level = (uint8_t)(kDepth - (31 - __clz(size)));
-            rs->s->t = t_in;
-            rs->s->nseg = (uint32_t)step;
-            return kSuspended;
-        }
-        if (UNIFORM) {
-#pragma unroll
-            for (int b = 0; b < 3; b++) lo[b] = ci[b] << ush;
-        }
-        double tb[3];
-        double t_out = __longlong_as_double(0x7ff0000000000000ll);
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            tb[b] = __longlong_as_double(0x7ff0000000000000ll);
-            if (d.flags & (1 << b)) {
-                const uint32_t F = (d.flags & (8 << b)) ? lo[b] + size : lo[b];
-                const double Fd = __dmul_rn(__uint2double_rn(F), 0x1p-21);
-                tb[b] = __dmul_rn(__dsub_rn(Fd, Q[b]), d.inv[b]);
-                t_out = fmin(t_out, tb[b]);
-            }
-        }
-        const double ds = __dsub_rn(t_out, t_in);
-        vis.seg((uint32_t)j, ds);
-        wc.nseg++;
-        t_in = t_out;
-        bool leaving = false;
-        unsigned E = 0;
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            if ((d.flags & (1 << b)) && tb[b] == t_out) {
-                E |= 1u << b;
-                if (d.flags & (8 << b)) {
-                    if (lo[b] + size >= t.ext[b]) leaving = true;
-                } else {
-                    if (lo[b] == 0) leaving = true;
-                }
-            }
-        }
-        if (leaving) break;
-        if (UNIFORM) {
-            // a non-stepped axis stays in its slab, which the neighbour shares
-#pragma unroll
-            for (int b = 0; b < 3; b++) {
-                if (E & (1u << b)) {
-                    const uint32_t mb = kDilX << b;
-                    uint32_t db = dil & mb;
-                    if (d.flags & (8 << b)) { ci[b]++; db = ((db | ~mb) + (1u << b)) & mb; }
-                    else { ci[b]--; db = (db - (1u << b)) & mb; }
-                    dil = (dil & ~mb) | db;
-                }
-            }
-            j = dil;
-        } else {
-            // The exit axes step; the others first take the leaf's lower
-            // corner.  Unless the leaf found there is finer than the current
-            // one it holds the whole face-adjacent cell of the current size
-            // (octree cells are aligned), hence the exit point: only a finer
-            // neighbour needs the position of the definition.
-#pragma unroll
-            for (int b = 0; b < 3; b++)
-                c[b] = (E & (1u << b)) ? ((d.flags & (8 << b)) ? lo[b] + size : lo[b] - 1) : lo[b];
-            uint64_t key;
-            int level;
-            j = lookup_leaf(t, c[0], c[1], c[2], key, level);
-            if (E != 7u && j >= 0 && (1u << (kDepth - level)) < size) {
-#pragma unroll
-                for (int b = 0; b < 3; b++) {
-                    if (!(E & (1u << b))) {
-                        const double P = __dadd_rn(Q[b], __dmul_rn(t_out, d.m[b]));
-                        double f = floor(__dmul_rn(P, 0x1p21));
-                        f = fmax(f, (double)lo[b]);
-                        f = fmin(f, (double)(lo[b] + size - 1));
-                        c[b] = (uint32_t)f;
-                    }
-                }
-                j = lookup_leaf(t, c[0], c[1], c[2], key, level);
-            }
-            if (j < 0) return RT_ERR_LOOKUP_MISS;
-            leaf_box(key, level, lo, size);
-        }
-    }
-    return RT_OK;
-}
 
 // FP64 walk on a full cube of equal-level leaves, moving axes VM (compile
 // time), in the mirrored frame of the F32-Kahan grid walk (a moving axis with
@@ -1162,8 +981,8 @@ static __device__ __noinline__ uint64_t find_leaf_packed(const DevTree t, uint64
     return find_leaf(t, x, j, ls) ? table_entry(j, ls) : ~0ull;
 }
 
-// Walk of one ray through a general octree, F32-Kahan arithmetic, moving axes
-// VM (compile time), in the mirrored frame of walk_f32k_grid: a moving axis
+// Walk of one ray through a general octree, moving axes VM (compile time), exit
+// decisions in certified FP32, in the mirrored frame of walk_f32k_grid: a moving axis
 // with m_b < 0 is reflected (cell c -> 2^21 - 1 - c = c ^ (2^21 - 1), and a
 // source integer qi -> 2^21 - qi), so that every exit face is the upper one,
 // at hi_b, every distance, reciprocal and time is positive, and a step needs
@@ -1181,9 +1000,15 @@ static __device__ __noinline__ uint64_t find_leaf_packed(const DevTree t, uint64
 // cells to spare on each side, more than the position's error; else (one step
 // in a thousand at leaves of 4096 lattice cells) near_point decides.
 //
-// Bound: instruction issue.
-template <int VM, bool QZ, class V, class R = NoResume>
-__device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* __restrict__ dp,
+// F64 (the FP64 form): only the exit axis's time is formed in FP64, as
+// fl(D (|inv| 2^-53)) with D = |F - Q| 2^53 an exact integer: F - Q is exact on the
+// 2^-53 lattice and the scaling by 2^-53 is exact, so it rounds the same real
+// product as the definition's fl((F - Q) inv) and gives the same double; ds is
+// their difference in FP64.
+//
+// Bound: instruction issue (the FP64 form at many species: the FP64 pipe).
+template <int VM, bool QZ, bool F64, class V, class R = NoResume>
+__device__ __forceinline__ int walk_tree(const DevTree& t, const DirConst* __restrict__ dp,
                                               const double* __restrict__ src, long long cap, V& vis,
                                               WalkCounters& wc, R* rs = nullptr)
 {
@@ -1196,6 +1021,7 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
     // lengths
     float ph[3], pl[3], qif[3], ihs[3];
     uint32_t hi[3], c[3];  // c: mirrored point
+    uint32_t qf[3];        // source fraction (2^-32 of a lattice cell)
     float cE = 0.f;
     // all ones on a reflected axis
     auto mir = [&](int b) { return (uint32_t)(__float_as_int(ihs[b]) >> 31); };
@@ -1203,11 +1029,11 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
     auto lower = [&](int b, uint32_t sz) { return mir(b) ? (1u << kDepth) - hi[b] : hi[b] - sz; };  // unreflected
     {
         int qi[3];
-        uint32_t qf[3];
         const int st = source_fixed(src, t, qi, qf, ph, pl);
         if (st != RT_OK) return st;
 #pragma unroll
         for (int b = 0; b < 3; b++) {
+            if (QZ) qf[b] = 0u;
             ihs[b] = (VM & (1 << b)) ? __ldg(&dp->ih[b]) * 0x1p-21f : 0.f;
             const bool neg = mir(b) != 0u;
             c[b] = ((uint32_t)qi[b] ^ mir(b)) & kOnes;
@@ -1222,6 +1048,7 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
     }
     uint32_t j, size;
     float tih = 0.f, til = 0.f;
+    double tin = 0.0;
     if (R::enabled && rs->s->status == 1) {
         j = rs->s->j;
         size = 1u << (kDepth - rs->s->level);
@@ -1229,6 +1056,7 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
         for (int b = 0; b < 3; b++) hi[b] = mir(b) ? (1u << kDepth) - rs->s->lo[b] : rs->s->lo[b] + size;
         tih = rs->s->th;
         til = rs->s->tl;
+        if (F64) tin = rs->s->t;
     } else {
         uint32_t x[3], ls;
 #pragma unroll
@@ -1248,6 +1076,7 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
             rs->s->level = (uint8_t)(kDepth - (31 - __clz(size)));
             rs->s->th = tih;
             rs->s->tl = til;
+            if (F64) rs->s->t = tin;
             rs->s->nseg = wc.nseg;
             return kSuspended;
         }
@@ -1284,7 +1113,7 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
             }
             if (near) {
                 const unsigned E = near_exit<VM, QZ>(t, dp, src, Af[0], Af[1], Af[2], th[0], th[1], th[2], cE);
-                wc.exit_fb += E >> 3;
+                if (!F64) wc.exit_fb += E >> 3;
 #pragma unroll
                 for (int b = 0; b < 3; b++) e[b] = (E >> b) & 1u;
             }
@@ -1293,25 +1122,40 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
         // A an integer, 0 or at least |ph|: (A - s) - ph is the rounding error
         const float Ae = e[0] ? Af[0] : (e[1] ? Af[1] : Af[2]);
         const float ihe = e[0] ? ihs[0] : (e[1] ? ihs[1] : ihs[2]);
-        const float* ilp = e[0] ? &dp->il[0] : (e[1] ? &dp->il[1] : &dp->il[2]);
-        const float ila = __ldg(ilp) * 0x1p-21f;
-        const float ile = __int_as_float(__float_as_int(ila) ^ (__float_as_int(ihe) & (int)0x80000000));
-        float the, tle;
-        if (QZ) {
-            the = __fmul_rn(Ae, fabsf(ihe));
-            tle = __fmaf_rn(Ae, ile, __fmaf_rn(Ae, fabsf(ihe), -the));
+        float the;
+        if (F64) {
+            the = t1;
+#pragma unroll
+            for (int b = 2; b >= 0; b--)
+                if (e[b]) the = th[b];
+            const double inv = fabs(__ldg(e[0] ? &dp->inv[0] : (e[1] ? &dp->inv[1] : &dp->inv[2])));
+            const double inv53 = __hiloint2double(__double2hiint(inv) - (53 << 20), __double2loint(inv));  // inv >= 1
+            const long long hi32 = (long long)small_float_to_int(Ae) << 32;
+            const long long fr = QZ ? 0ll : (long long)(e[0] ? qf[0] : (e[1] ? qf[1] : qf[2]));
+            const double tout = __dmul_rn(__ll2double_rn(ihe < 0.f ? hi32 + fr : hi32 - fr), inv53);
+            vis.acc(__dsub_rn(tout, tin));
+            tin = tout;
         } else {
-            const float se = e[0] ? sd[0] : (e[1] ? sd[1] : sd[2]);
-            const float pe = e[0] ? ph[0] : (e[1] ? ph[1] : ph[2]);
-            const float le = e[0] ? pl[0] : (e[1] ? pl[1] : pl[2]);
-            const float rl = __fsub_rn(__fsub_rn(__fsub_rn(Ae, se), pe), le);
-            the = __fmul_rn(se, fabsf(ihe));
-            tle = __fadd_rn(__fmaf_rn(se, fabsf(ihe), -the), __fmaf_rn(se, ile, __fmul_rn(rl, fabsf(ihe))));
+            const float* ilp = e[0] ? &dp->il[0] : (e[1] ? &dp->il[1] : &dp->il[2]);
+            const float ila = __ldg(ilp) * 0x1p-21f;
+            const float ile = __int_as_float(__float_as_int(ila) ^ (__float_as_int(ihe) & (int)0x80000000));
+            float tle;
+            if (QZ) {
+                the = __fmul_rn(Ae, fabsf(ihe));
+                tle = __fmaf_rn(Ae, ile, __fmaf_rn(Ae, fabsf(ihe), -the));
+            } else {
+                const float se = e[0] ? sd[0] : (e[1] ? sd[1] : sd[2]);
+                const float pe = e[0] ? ph[0] : (e[1] ? ph[1] : ph[2]);
+                const float le = e[0] ? pl[0] : (e[1] ? pl[1] : pl[2]);
+                const float rl = __fsub_rn(__fsub_rn(__fsub_rn(Ae, se), pe), le);
+                the = __fmul_rn(se, fabsf(ihe));
+                tle = __fadd_rn(__fmaf_rn(se, fabsf(ihe), -the), __fmaf_rn(se, ile, __fmul_rn(rl, fabsf(ihe))));
+            }
+            const float ds = __fadd_rn(__fsub_rn(the, tih), __fsub_rn(tle, til));
+            tih = the;
+            til = tle;
+    vis.acc(ds);
         }
-        const float ds = __fadd_rn(__fsub_rn(the, tih), __fsub_rn(tle, til));
-        tih = the;
-        til = tle;
-        vis.acc(ds);
         wc.nseg++;
         // the exit axes enter the next cell, the others take the exit point; a
         // fixed coordinate stays inside every leaf on the path
@@ -1356,7 +1200,7 @@ __device__ __forceinline__ int walk_f32k_tree(const DevTree& t, const DirConst* 
                 for (int b = 0; b < 3; b++) x[b] = (c[b] ^ mir(b)) & kOnes;
                 const uint64_t p = near_point<VM, QZ>(t, dp, src, E, the, Ae, x[0], x[1], x[2], lower(0, size0),
                                                       lower(1, size0), lower(2, size0), size0);
-                wc.lookup_fb += (uint32_t)(p >> 63);
+                if (!F64) wc.lookup_fb += (uint32_t)(p >> 63);
                 const uint64_t found = find_leaf_packed(t, p);
                 hit = found != ~0ull;
                 j = (uint32_t)found;
@@ -1407,35 +1251,19 @@ __device__ __forceinline__ int walk_grid_vm(int vm, const DevTree& t, const DirC
     }
 }
 
-template <bool QZ, class V>
+template <bool QZ, bool F64, class V, class R = NoResume>
 __device__ __forceinline__ int walk_tree_vm(int vm, const DevTree& t, const DirConst* __restrict__ dp,
                                             const double* __restrict__ src, long long cap, V& vis,
-                                            WalkCounters& wc)
+                                            WalkCounters& wc, R* rs = nullptr)
 {
     switch (vm) {
-    case 1: return walk_f32k_tree<1, QZ>(t, dp, src, cap, vis, wc);
-    case 2: return walk_f32k_tree<2, QZ>(t, dp, src, cap, vis, wc);
-    case 3: return walk_f32k_tree<3, QZ>(t, dp, src, cap, vis, wc);
-    case 4: return walk_f32k_tree<4, QZ>(t, dp, src, cap, vis, wc);
-    case 5: return walk_f32k_tree<5, QZ>(t, dp, src, cap, vis, wc);
-    case 6: return walk_f32k_tree<6, QZ>(t, dp, src, cap, vis, wc);
-    default: return walk_f32k_tree<7, QZ>(t, dp, src, cap, vis, wc);
-    }
-}
-
-template <bool QZ, class V, class R>
-__device__ __forceinline__ int walk_tree_vm_r(int vm, const DevTree& t, const DirConst* __restrict__ dp,
-                                              const double* __restrict__ src, long long cap, V& vis,
-                                              WalkCounters& wc, R* rs)
-{
-    switch (vm) {
-    case 1: return walk_f32k_tree<1, QZ>(t, dp, src, cap, vis, wc, rs);
-    case 2: return walk_f32k_tree<2, QZ>(t, dp, src, cap, vis, wc, rs);
-    case 3: return walk_f32k_tree<3, QZ>(t, dp, src, cap, vis, wc, rs);
-    case 4: return walk_f32k_tree<4, QZ>(t, dp, src, cap, vis, wc, rs);
-    case 5: return walk_f32k_tree<5, QZ>(t, dp, src, cap, vis, wc, rs);
-    case 6: return walk_f32k_tree<6, QZ>(t, dp, src, cap, vis, wc, rs);
-    default: return walk_f32k_tree<7, QZ>(t, dp, src, cap, vis, wc, rs);
+    case 1: return walk_tree<1, QZ, F64>(t, dp, src, cap, vis, wc, rs);
+    case 2: return walk_tree<2, QZ, F64>(t, dp, src, cap, vis, wc, rs);
+    case 3: return walk_tree<3, QZ, F64>(t, dp, src, cap, vis, wc, rs);
+    case 4: return walk_tree<4, QZ, F64>(t, dp, src, cap, vis, wc, rs);
+    case 5: return walk_tree<5, QZ, F64>(t, dp, src, cap, vis, wc, rs);
+    case 6: return walk_tree<6, QZ, F64>(t, dp, src, cap, vis, wc, rs);
+    default: return walk_tree<7, QZ, F64>(t, dp, src, cap, vis, wc, rs);
     }
 }
 
@@ -1448,13 +1276,10 @@ __device__ __forceinline__ int walk_chunk(const DevTree& t, const DirConst* __re
                                           const double* __restrict__ src, long long cap, V& vis,
                                           WalkCounters& wc, ChunkResume* rs)
 {
-    if (MODE == RT_MODE_FP64) {
-        const DirConst d = *dp;
-        return walk_fp64<false>(t, d, src, cap, vis, wc, rs);
-    }
+    constexpr bool F64 = MODE == RT_MODE_FP64;
     const int vm = __ldg(&dp->flags) & 7;
-    return source_on_lattice(src) ? walk_tree_vm_r<true>(vm, t, dp, src, cap, vis, wc, rs)
-                                  : walk_tree_vm_r<false>(vm, t, dp, src, cap, vis, wc, rs);
+    return source_on_lattice(src) ? walk_tree_vm<true, F64>(vm, t, dp, src, cap, vis, wc, rs)
+                                  : walk_tree_vm<false, F64>(vm, t, dp, src, cap, vis, wc, rs);
 }
 
 // Walk of one ray (direction *dp, in global memory) in either arithmetic form.
@@ -1463,31 +1288,28 @@ __device__ __forceinline__ int walk(const DevTree& t, const DirConst* __restrict
                                     const double* __restrict__ src, long long cap, V& vis,
                                     WalkCounters& wc)
 {
-    if (MODE == RT_MODE_FP64) {
-        if (UNIFORM) {
-            const int fl = __ldg(&dp->flags);
-            if (((fl & 7) == 3 || (fl & 7) == 7) && xy_locked_fp64(t, fl, src)) {
-                if ((fl & 7) == 3) return walk_fp64_grid<3, true>(t, dp, src, cap, vis, wc);
-                return walk_fp64_grid<7, true>(t, dp, src, cap, vis, wc);
-            }
-            switch (fl & 7) {
-            case 1: return walk_fp64_grid<1, false>(t, dp, src, cap, vis, wc);
-            case 2: return walk_fp64_grid<2, false>(t, dp, src, cap, vis, wc);
-            case 3: return walk_fp64_grid<3, false>(t, dp, src, cap, vis, wc);
-            case 4: return walk_fp64_grid<4, false>(t, dp, src, cap, vis, wc);
-            case 5: return walk_fp64_grid<5, false>(t, dp, src, cap, vis, wc);
-            case 6: return walk_fp64_grid<6, false>(t, dp, src, cap, vis, wc);
-            default: return walk_fp64_grid<7, false>(t, dp, src, cap, vis, wc);
-            }
+    if (UNIFORM && MODE == RT_MODE_FP64) {
+        const int fl = __ldg(&dp->flags);
+        if (((fl & 7) == 3 || (fl & 7) == 7) && xy_locked_fp64(t, fl, src)) {
+            if ((fl & 7) == 3) return walk_fp64_grid<3, true>(t, dp, src, cap, vis, wc);
+            return walk_fp64_grid<7, true>(t, dp, src, cap, vis, wc);
         }
-        const DirConst d = *dp;
-        return walk_fp64<UNIFORM>(t, d, src, cap, vis, wc);
+        switch (fl & 7) {
+        case 1: return walk_fp64_grid<1, false>(t, dp, src, cap, vis, wc);
+        case 2: return walk_fp64_grid<2, false>(t, dp, src, cap, vis, wc);
+        case 3: return walk_fp64_grid<3, false>(t, dp, src, cap, vis, wc);
+        case 4: return walk_fp64_grid<4, false>(t, dp, src, cap, vis, wc);
+        case 5: return walk_fp64_grid<5, false>(t, dp, src, cap, vis, wc);
+        case 6: return walk_fp64_grid<6, false>(t, dp, src, cap, vis, wc);
+        default: return walk_fp64_grid<7, false>(t, dp, src, cap, vis, wc);
+        }
     }
     const int vm = __ldg(&dp->flags) & 7;
     const bool qz = source_on_lattice(src);
     if (UNIFORM)
         return qz ? walk_grid_vm<true>(vm, t, dp, src, cap, vis, wc) : walk_grid_vm<false>(vm, t, dp, src, cap, vis, wc);
-    return qz ? walk_tree_vm<true>(vm, t, dp, src, cap, vis, wc) : walk_tree_vm<false>(vm, t, dp, src, cap, vis, wc);
+    constexpr bool F64 = MODE == RT_MODE_FP64;
+    return qz ? walk_tree_vm<true, F64>(vm, t, dp, src, cap, vis, wc) : walk_tree_vm<false, F64>(vm, t, dp, src, cap, vis, wc);
 }
 
 // ------------------------------------------------------------- densities

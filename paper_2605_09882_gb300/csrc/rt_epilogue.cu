@@ -95,6 +95,7 @@ extern "C" int rt_trace_epilogue(const rt_octree* t, const double* d_src, int64_
     cudaGetDevice(&dev);
     const int fit = occupancy_epi(mode, n_species, a.t.uniform_level >= 0, block);
     const int grid = sm_count_of(dev) * std::max(1, bps > 0 ? std::min(bps, fit) : fit);
+    spread_rays(a, (long long)grid * (block / 32));
     if (cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess ||
         launch_epilogue(a, mode, block, grid, s) != cudaSuccess)
         return cuda_error("rt_trace_epilogue: launch");

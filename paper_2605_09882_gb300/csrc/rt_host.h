@@ -16,6 +16,9 @@ void launch_shape(int* block, int* blocks_per_sm, int* groups_per_pop);
 // device direction table of nside on device dev (uploaded on first use)
 const DirConst* direction_table(int dev, int nside, int* status);
 int sm_count_of(int dev);
+// spreads a call of few rays over the warps of its launch (groups per pop, rays
+// per group)
+void spread_rays(TraceArgs& a, long long warps);
 // deepest coarse-table level rt_build_octree may choose (-1: no cap)
 int table_level_cap();
 // enqueues the density check (RT_ERR_NONFINITE into st for a NaN, infinite or

@@ -75,7 +75,8 @@ struct TraceArgs {
     uint32_t* nseg;          // path fingerprints (optional)
     uint64_t* hash;
     DevStats* st;
-    int batch;               // 32-ray groups per queue pop
+    int batch;               // ray groups per queue pop
+    int gw;                  // rays a group: 32, or fewer to spread a call of few rays over the warps
     int layout;              // ray order: 0 direction-major (sources padded to 32), 1 source-major
     int dgroup;              // layout 0: directions per group (a power of two dividing nd; <= 1: one)
     int pair;                // forward on a uniform cube: two rays per lane (k_trace_pair; n_src_pad % 64 == 0),

@@ -1,4 +1,5 @@
-// Persistent trace kernels: a warp pops 32 * batch consecutive rays from
+// Persistent trace kernels: a warp pops gw * batch (gw: 32, fewer for a call of
+// few rays) consecutive rays from
 // a global counter (one atomic per pop, no waiting), each lane walks one ray.
 // Ray r of the padded space maps direction-major: q = r / n_src_pad,
 // s = r % n_src_pad, so a warp walks 32 neighbouring sources (Morton order)
@@ -16,6 +17,9 @@
 #endif
 #ifndef RT_MIN_BLOCKS_TREE
 #define RT_MIN_BLOCKS_TREE 4
+#endif
+#ifndef RT_MIN_BLOCKS_F64TREE
+#define RT_MIN_BLOCKS_F64TREE 2
 #endif
 #ifndef RT_MIN_BLOCKS
 #define RT_MIN_BLOCKS 1
@@ -236,7 +240,7 @@ __device__ __forceinline__ void forward_ray(const TraceArgs& a, const DirConst* 
 
 template <int KIND, int MODE, bool UNIFORM, int SM>
 __global__ void __launch_bounds__(256, (MODE == RT_MODE_F32_KAHAN) ? (UNIFORM ? RT_MIN_BLOCKS_GRID : RT_MIN_BLOCKS_TREE)
-                                                                : RT_MIN_BLOCKS)
+                                                                : (UNIFORM ? RT_MIN_BLOCKS : RT_MIN_BLOCKS_F64TREE))
 k_trace(const TraceArgs a)
 {
     // the shared-offset form ran before: only the sources it left out, if any
@@ -244,20 +248,22 @@ k_trace(const TraceArgs a)
     if (UNIFORM && a.pair && !rest) return;  // k_trace_pair traced every source
     const unsigned n_rest = rest && a.n_rest ? *(volatile const unsigned*)a.n_rest : 0u;
     if (rest && n_rest == 0u) return;
-    if (MODE == RT_MODE_F32_KAHAN && !UNIFORM) fill_spread_table();
+    if (!UNIFORM) fill_spread_table();
     const int lane = threadIdx.x & 31;
+    const int gw = KIND == 3 ? 32 : a.gw;  // rays a warp walks at once
     const unsigned long long rest_pad = (n_rest + 31u) & ~31u;
     const unsigned long long total = (rest ? rest_pad : (unsigned long long)(a.layout ? a.n_src : a.n_src_pad)) * (unsigned long long)a.nd;
     const long long cap = a.t.step_cap;
     unsigned long long n_rays = 0, n_segs = 0, n_efb = 0, n_lfb = 0;
     for (;;) {
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&a.st->queue, 32ull * (unsigned)a.batch);
+        if (lane == 0) base = atomicAdd(&a.st->queue, (unsigned long long)gw * (unsigned)a.batch);
         base = __shfl_sync(RT_FULL, base, 0);
         if (base >= total) break;
         for (int kk = 0; kk < a.batch; kk++) {
-            const unsigned long long g0 = base + 32ull * kk;
+            const unsigned long long g0 = base + (unsigned long long)gw * kk;
             if (g0 >= total) break;
+            if (lane >= gw) continue;
             int q;
             long long s;
             if (rest) {

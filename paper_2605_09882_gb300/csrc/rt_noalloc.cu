@@ -181,10 +181,12 @@ extern "C" int rt_trace_columns_noalloc(const uint64_t* d_keys, const uint8_t* d
     int block, bps, groups;
     launch_shape(&block, &bps, &groups);
     a.batch = groups;
+    a.gw = 32;
     a.layout = ray_layout(n_src);
     if (n_src > 0) {
         const int fit = std::max(1, occupancy_fwd(0, mode, n_species, uniform, block));
         const int per_sm = bps > 0 ? std::min(bps, fit) : fit;
+        spread_rays(a, (long long)sm_count_of(dev) * per_sm * (block / 32));
         if (launch_forward(a, mode, block, sm_count_of(dev) * per_sm, s) != cudaSuccess)
             return cuda_error("rt_trace_columns_noalloc: launch");
     }

@@ -109,3 +109,29 @@ def test_captured_call_walks(rt):
     torch.cuda.synchronize()
     assert torch.equal(out, want)
     tree.close()
+
+
+@pytest.mark.parametrize("n_src,nside", [(1, 1), (1, 8), (7, 4), (31, 2), (33, 1), (100, 2)])
+@pytest.mark.parametrize("mode", ["f32k", "fp64"])
+def test_few_rays_equal_many(rt, n_src, nside, mode):
+    """A call of few rays gives each warp fewer than 32 of them; the columns,
+    the gradient's terms and the paths are those of the same sources among many."""
+    import torch
+    from tinytrees import random_octree
+    rng = np.random.default_rng(77)
+    keys, lev, _ = random_octree(rng, 1, 6, 0.35)
+    tree = rt.Octree(_dev(keys), _dev(lev))
+    dens = _dev(rng.random((keys.shape[0], 3)).astype(np.float32))
+    many = _dev(rng.random((6000, 3)))
+    few = many[:n_src]
+    want = rt.trace_columns(tree, many, nside, dens, mode)[:n_src]
+    assert torch.equal(rt.trace_columns(tree, few, nside, dens, mode), want)
+    for a, b in zip(rt.trace_paths(tree, few, nside, mode), rt.trace_paths(tree, many, nside, mode)):
+        assert torch.equal(a, b[:n_src])
+    # the transpose of the columns: <g, A n> = <A^T g, n>, FP64 sums of
+    # non-negative terms against FP32 columns within their 1e-5
+    g = torch.rand(want.shape, device="cuda", dtype=want.dtype)
+    grad = rt.trace_columns_adjoint(tree, few, nside, g, mode)
+    lhs, rhs = (g.double() * want.double()).sum(), (grad * dens.double()).sum()
+    torch.testing.assert_close(lhs, rhs, rtol=1e-12 if mode == "fp64" else 1e-5, atol=0)
+    tree.close()
