@@ -124,25 +124,44 @@ extern "C" int rt_build_amr(const void* d_nref, int nref_dtype, const void* d_va
     uint8_t* lvl = nullptr;
     int* start = nullptr;
     long long* pos = nullptr;
-    void* tmp = nullptr;
-    size_t tmp_bytes = 0;
+    char* scratch = nullptr;
+    size_t tmp_bytes = 0, at = 0, tmp_at = 0;
     int status = RT_OK;
     long long last_pos = 0;
     int last_start = 0;
     PyrPtrs pp;
     memset(&pp, 0, sizeof pp);
-    for (int l = 0; l < L; l++) {
-        const long long nc = 1ll << (3 * l);
-        if (cudaMalloc(&mn[l], sizeof(double) * nc) != cudaSuccess || cudaMalloc(&mx[l], sizeof(double) * nc) != cudaSuccess ||
-            cudaMalloc(&sum[l], sizeof(double) * nc * S) != cudaSuccess || cudaMalloc(&split[l], nc) != cudaSuccess) {
-            status = set_error(RT_ERR_OOM, "rt_build_amr: pyramid allocation");
+    // one block for the pyramid, the per-cell arrays and the scan's scratch (an
+    // allocation for each of them, and its release, cost more than the kernels)
+    if (cub::DeviceScan::ExclusiveSum(nullptr, tmp_bytes, start, pos, n, s) != cudaSuccess) {
+        status = cuda_error("rt_build_amr: scan");
+        goto done;
+    }
+    for (int pass = 0; pass < 2; pass++) {  // sizes, then addresses
+        at = 0;
+        auto take = [&](size_t bytes) {
+            void* p = scratch ? scratch + at : nullptr;
+            at += (bytes + 255) / 256 * 256;
+            return p;
+        };
+        for (int l = 0; l < L; l++) {
+            const long long nc = 1ll << (3 * l);
+            mn[l] = (double*)take(sizeof(double) * nc);
+            mx[l] = (double*)take(sizeof(double) * nc);
+            sum[l] = (double*)take(sizeof(double) * nc * S);
+            split[l] = (uint8_t*)take(nc);
+        }
+        lvl = (uint8_t*)take(n);
+        start = (int*)take(sizeof(int) * n);
+        pos = (long long*)take(sizeof(long long) * n);
+        tmp_at = at;
+        take(tmp_bytes);
+        if (pass == 0 && cudaMalloc(&scratch, at) != cudaSuccess) {
+            cudaGetLastError();
+            scratch = nullptr;
+            status = set_error(RT_ERR_OOM, "rt_build_amr: allocation");
             goto done;
         }
-    }
-    if (cudaMalloc(&lvl, n) != cudaSuccess || cudaMalloc(&start, sizeof(int) * n) != cudaSuccess ||
-        cudaMalloc(&pos, sizeof(long long) * n) != cudaSuccess) {
-        status = set_error(RT_ERR_OOM, "rt_build_amr: allocation");
-        goto done;
     }
     for (int l = L - 1; l >= 0; l--) {
         const long long nc = 1ll << (3 * l);
@@ -159,12 +178,7 @@ extern "C" int rt_build_amr(const void* d_nref, int nref_dtype, const void* d_va
     {
         const int grid = (int)std::min<long long>((n + 255) / 256, gmax);
         k_leaf_levels<<<grid, 256, 0, s>>>(L, n, pp, lvl, start);
-        cub::DeviceScan::ExclusiveSum(nullptr, tmp_bytes, start, pos, n, s);
-        if (cudaMalloc(&tmp, tmp_bytes) != cudaSuccess) {
-            status = set_error(RT_ERR_OOM, "rt_build_amr: scan scratch");
-            goto done;
-        }
-        cub::DeviceScan::ExclusiveSum(tmp, tmp_bytes, start, pos, n, s);
+        cub::DeviceScan::ExclusiveSum(scratch + tmp_at, tmp_bytes, start, pos, n, s);
         k_emit<<<grid, 256, 0, s>>>(L, n, pp, d_nref, nref_dtype == RT_F64, d_vals, vals_dtype == RT_F64, S, lvl, start,
                                     pos, d_keys, d_levels, d_leaf_vals, vals_dtype == RT_F64);
         cudaMemcpyAsync(&last_pos, pos + (n - 1), sizeof last_pos, cudaMemcpyDeviceToHost, s);
@@ -176,16 +190,7 @@ extern "C" int rt_build_amr(const void* d_nref, int nref_dtype, const void* d_va
         *h_n_leaves = last_pos + last_start;
     }
 done:
-    for (int l = 0; l < L; l++) {
-        if (mn[l]) cudaFree(mn[l]);
-        if (mx[l]) cudaFree(mx[l]);
-        if (sum[l]) cudaFree(sum[l]);
-        if (split[l]) cudaFree(split[l]);
-    }
-    if (lvl) cudaFree(lvl);
-    if (start) cudaFree(start);
-    if (pos) cudaFree(pos);
-    if (tmp) cudaFree(tmp);
+    if (scratch) cudaFree(scratch);
     if (status == RT_OK) clear_error();
     return status;
 }

@@ -837,6 +837,19 @@ __device__ __forceinline__ int floor_small(float v)
     return __float_as_int(__fadd_rd(v, 12582912.0f)) - 0x4B400000;
 }
 
+// First leaf and code of a coarse cell.
+__device__ __forceinline__ uint32_t table_cell(const DevTree& t, uint32_t cell, uint32_t& code)
+{
+    if (t.wide) {
+        const uint2 e = __ldg((const uint2*)t.table + cell);
+        code = e.y;
+        return e.x;
+    }
+    const uint32_t e = __ldg((const uint32_t*)t.table + cell);
+    code = e & 63u;
+    return e >> 6;
+}
+
 // The rarer kinds of coarse cell, out of line (the octree by value: a reference
 // would put the caller's into local memory): leaves two or more levels below the table, and a mixed cell, searched
 // by key.  Leaf in the low half, log2 of its size in the high one; all ones: no
@@ -853,7 +866,8 @@ static __device__ __noinline__ uint64_t find_in_cell(const DevTree t, uint32_t x
     if (code == kCellHole) return ~0ull;
     const uint64_t M = interleave3(x, y, z);
     const uint32_t ncell = 1u << (3 * t.T);
-    long long hi = cell + 1 < ncell ? (long long)__ldg((const uint2*)t.table + cell + 1).x : t.n;
+    uint32_t next;
+    long long hi = cell + 1 < ncell ? (long long)table_cell(t, cell + 1, next) : t.n;
     long long lo = (long long)first;  // keys[lo] == cell base <= M
     while (hi - lo > 1) {
         const long long mid = (lo + hi) >> 1;
@@ -874,16 +888,17 @@ __device__ __forceinline__ bool find_leaf(const DevTree& t, const uint32_t c[3],
     const uint32_t tmask = (1u << t.T) - 1u;  // T <= 10: inside the spread table
     const uint32_t cell = s_spread10[(c[0] >> s) & tmask] + 2u * s_spread10[(c[1] >> s) & tmask] +
                           4u * s_spread10[(c[2] >> s) & tmask];
-    const uint2 e = __ldg((const uint2*)t.table + cell);
-    j = e.x;
-    ls = e.y;
-    if (e.y < kCellLeaves) return true;
-    ls = e.y - kCellLeaves;
+    uint32_t code;
+    const uint32_t first = table_cell(t, cell, code);
+    j = first;
+    ls = code;
+    if (code < kCellLeaves) return true;
+    ls = code - kCellLeaves;
     if ((int)ls + 1 == s) {  // one level below the table: the octant
         j += ((c[0] >> ls) & 1u) + 2u * ((c[1] >> ls) & 1u) + 4u * ((c[2] >> ls) & 1u);
         return true;
     }
-    const uint64_t found = find_in_cell(t, c[0], c[1], c[2], cell, e.x, e.y);
+    const uint64_t found = find_in_cell(t, c[0], c[1], c[2], cell, first, code);
     j = (uint32_t)found;
     ls = (uint32_t)(found >> 32) & 31u;
     return found != ~0ull;

@@ -12,24 +12,28 @@ constexpr int kDepth = 21;          // anchor depth of the Morton lattice
 constexpr int kMaxSpecies = 8;
 constexpr int kBaseTableLevel = 7;  // coarse table level for every tree (8^7 = 2M entries at most)
 constexpr int kMaxTableLevel = 10;  // deepest coarse table (the lookup's cell index holds 30 bits)
-// Coarse-table entries: the first leaf in the low half, in the high half what
-// is there: log2 of the leaf's size for a cell inside one leaf, kCellLeaves
-// more than that for a cell whose leaves all have one finer level, or one of
-// the two codes after it.  Whole halves, so that a lookup takes neither without
-// a 64-bit shift.
+// Coarse-table entries: the first leaf and a code for what is there: log2 of the
+// leaf's size for a cell inside one leaf, kCellLeaves more than that for a cell
+// whose leaves all have one finer level, or one of the two codes after it.
+// An octree of fewer than 2^26 leaves packs them into 32 bits, leaf << 6 | code:
+// at level 8 the table then takes 67 MB, beside the leaves' densities in a 129
+// MB L2, and not 134.  A larger one keeps the leaf in the low half of 64 bits and
+// the code in the high half.
 constexpr uint32_t kCellLeaves = 32;
-constexpr uint32_t kCellMixed = 64;  // leaves of several levels
-constexpr uint32_t kCellHole = 65;   // outside the domain box
+constexpr uint32_t kCellMixed = 62;  // leaves of several levels
+constexpr uint32_t kCellHole = 63;   // outside the domain box
+constexpr int64_t kNarrowLeaves = 1ll << 26;
 constexpr uint64_t table_entry(uint64_t first, uint32_t code) { return first | (uint64_t)code << 32; }
 
 // Device view of an octree handle.
 struct DevTree {
     const uint64_t* keys;
     const uint8_t* levels;
-    const uint64_t* table;   // [8^T] entries (table_entry)
+    const void* table;       // [8^T] entries, uint32 or (wide) uint64
     int64_t n;
     uint32_t ext[3];
     int T;                   // coarse table level
+    int wide;                // 64-bit table entries
     int uniform_level;       // >= 0: full cube of leaves all at this level (O(1) index)
     int lmax;
     int64_t step_cap;
@@ -121,7 +125,7 @@ int occupancy_adj(int mode, int S, bool uniform, int block);
 struct rt_octree {
     rt::DevTree dev;
     rt::DevStats* st;        // device
-    uint64_t* table;         // device, owned
+    void* table;             // device, owned
     int device;
     int uniform_allowed;     // 0: use the coarse table even for a uniform grid
     int64_t default_cap;

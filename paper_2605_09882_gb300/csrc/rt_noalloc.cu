@@ -164,6 +164,7 @@ extern "C" int rt_trace_columns_noalloc(const uint64_t* d_keys, const uint8_t* d
     a.t.n = n_leaves;
     for (int b = 0; b < 3; b++) a.t.ext[b] = ext[b];
     a.t.T = 0;
+    a.t.wide = 1;
     a.t.uniform_level = uniform ? max_level : -1;
     a.t.lmax = max_level;
     a.t.step_cap = 3 * (1ll << max_level) + 3;

@@ -81,9 +81,9 @@ __global__ void k_cell_levels(const uint64_t* __restrict__ keys, const uint8_t* 
     }
 }
 
-__device__ __forceinline__ int64_t lower_bound_keys(const uint64_t* keys, int64_t n, uint64_t v)
+// First index in [lo, hi) whose key is at least v, hi if none.
+__device__ __forceinline__ int64_t lower_bound_keys(const uint64_t* keys, int64_t lo, int64_t hi, uint64_t v)
 {
-    int64_t lo = 0, hi = n;
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
         if (keys[mid] < v) lo = mid + 1;
@@ -98,16 +98,24 @@ __device__ __forceinline__ int64_t lower_bound_keys(const uint64_t* keys, int64_
 //                          local index;
 //   kCellMixed           : binary search in [first, next cell's first);
 //   kCellHole            : the cell starts outside the domain box.
+//
+// A warp's 32 cells are neighbours in key order: one search for the first of
+// them and one for their end, the same for every lane (one load a step), leave
+// each lane the few leaves between (a search of all keys by every lane is 24
+// dependent gathers at 10M leaves).
 __global__ void k_fill_table(const uint64_t* __restrict__ keys, const uint8_t* __restrict__ levels,
                              int64_t n, int T, uint32_t ex, uint32_t ey, uint32_t ez,
-                             const unsigned* lvmin, const unsigned* lvmax, uint64_t* table)
+                             const unsigned* lvmin, const unsigned* lvmax, void* table, int wide)
 {
     const int csh = 3 * (kDepth - T);
     const uint64_t ncell = 1ull << (3 * T);
     for (uint64_t C = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; C < ncell;
          C += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t base = C << csh;
-        const int64_t j0 = lower_bound_keys(keys, n, base);
+        const uint64_t W = C & ~31ull;
+        const int64_t w0 = lower_bound_keys(keys, 0, n, W << csh);
+        const int64_t w1 = W + 32 < ncell ? lower_bound_keys(keys, w0, n, (W + 32) << csh) : n;
+        const int64_t j0 = lower_bound_keys(keys, w0, w1, base);
         uint32_t code;
         int64_t first = j0;
         if (compact21(base) >= ex || compact21(base >> 1) >= ey || compact21(base >> 2) >= ez) {
@@ -119,12 +127,13 @@ __global__ void k_fill_table(const uint64_t* __restrict__ keys, const uint8_t* _
             code = kDepth - levels[j0];
         } else if (lvmin[C] == lvmax[C]) {
             const int l = (int)lvmin[C];
-            const int64_t j1 = lower_bound_keys(keys, n, base + (1ull << csh));
+            const int64_t j1 = lower_bound_keys(keys, j0, w1, base + (1ull << csh));
             code = (j1 - j0 == (int64_t)(1ull << (3 * (l - T)))) ? kCellLeaves + kDepth - l : kCellMixed;
         } else {
             code = kCellMixed;
         }
-        table[C] = table_entry((uint64_t)first, code);
+        if (wide) ((uint64_t*)table)[C] = table_entry((uint64_t)first, code);
+        else ((uint32_t*)table)[C] = (uint32_t)first << 6 | code;
     }
 }
 
@@ -202,7 +211,7 @@ extern "C" int rt_build_octree(const uint64_t* d_keys, const uint8_t* d_levels, 
     cudaGetDevice(&t->device);
     ValOut* vo = nullptr;
     ValOut hv;
-    unsigned *lvmin = nullptr, *lvmax = nullptr;
+    unsigned* lv = nullptr;  // level range of every coarse cell
     int status = RT_OK;
     const int blocks = (int)std::min<int64_t>((n_leaves + 255) / 256, 4096);
     if (cudaMalloc(&t->st, sizeof(DevStats)) != cudaSuccess || cudaMalloc(&vo, sizeof(ValOut)) != cudaSuccess) {
@@ -241,25 +250,25 @@ extern "C" int rt_build_octree(const uint64_t* d_keys, const uint8_t* d_levels, 
         const int cap = table_level_cap();
         if (cap >= 0) T = std::min(T, cap);
         const uint64_t ncell = 1ull << (3 * T);
-        if (cudaMalloc(&t->table, ncell * sizeof(uint64_t)) != cudaSuccess ||
-            cudaMalloc(&lvmin, ncell * sizeof(unsigned)) != cudaSuccess ||
-            cudaMalloc(&lvmax, ncell * sizeof(unsigned)) != cudaSuccess) {
+        const int wide = n_leaves >= kNarrowLeaves;
+        if (cudaMalloc(&t->table, ncell * (wide ? 8 : 4)) != cudaSuccess ||
+            cudaMalloc(&lv, 2 * ncell * sizeof(unsigned)) != cudaSuccess) {
             status = set_error(RT_ERR_OOM, "rt_build_octree: table allocation");
             goto fail;
         }
+        unsigned *lvmin = lv, *lvmax = lv + ncell;
         cudaMemsetAsync(lvmin, 0xff, ncell * sizeof(unsigned), s);
         cudaMemsetAsync(lvmax, 0, ncell * sizeof(unsigned), s);
         k_cell_levels<<<blocks, 256, 0, s>>>(d_keys, d_levels, n_leaves, T, lvmin, lvmax);
         const int cblocks = (int)std::min<uint64_t>((ncell + 255) / 256, 4096);
         k_fill_table<<<cblocks, 256, 0, s>>>(d_keys, d_levels, n_leaves, T, ext[0], ext[1], ext[2],
-                                             lvmin, lvmax, t->table);
+                                             lvmin, lvmax, t->table, wide);
         if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
             status = cuda_error("rt_build_octree: table build");
             goto fail;
         }
-        cudaFree(lvmin);
-        cudaFree(lvmax);
-        lvmin = lvmax = nullptr;
+        cudaFree(lv);
+        lv = nullptr;
         DevTree& d = t->dev;
         d.keys = d_keys;
         d.levels = d_levels;
@@ -267,6 +276,7 @@ extern "C" int rt_build_octree(const uint64_t* d_keys, const uint8_t* d_levels, 
         d.n = n_leaves;
         for (int b = 0; b < 3; b++) d.ext[b] = ext[b];
         d.T = T;
+        d.wide = wide;
         d.lmax = lmax;
         d.uniform_level = uniform ? lmax : -1;
         static std::atomic<unsigned long long> builds{0};
@@ -281,8 +291,7 @@ extern "C" int rt_build_octree(const uint64_t* d_keys, const uint8_t* d_levels, 
     return RT_OK;
 fail:
     if (vo) cudaFree(vo);
-    if (lvmin) cudaFree(lvmin);
-    if (lvmax) cudaFree(lvmax);
+    if (lv) cudaFree(lv);
     if (t->table) cudaFree(t->table);
     if (t->st) cudaFree(t->st);
     free(t);
