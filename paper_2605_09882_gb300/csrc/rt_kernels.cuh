@@ -10,8 +10,11 @@
 #include "rt_device.cuh"
 
 // Resident 256-thread blocks per SM the register budget is sized for: both
-// F32-Kahan walks run best at 64 registers (4 blocks); the FP64 walks keep
-// the compiler's choice.
+// F32-Kahan walks run best at 64 registers (4 blocks; the tree walk's A_V,eff on
+// a 64^3-base cloud 20.7 ms, at 3 blocks 22.8, at 2 26.5); the FP64 tree walk at
+// 128 (2 blocks; the same cloud's columns 7.4 ms, also at 3 and 4 blocks, which
+// spill, and 8.9 at the compiler's 255); the FP64 grid walk keeps the compiler's
+// choice.
 #ifndef RT_MIN_BLOCKS_GRID
 #define RT_MIN_BLOCKS_GRID 4
 #endif
