@@ -88,6 +88,8 @@ struct BeamTables {
     int* fb;         // [nd][lcap] exit fall-backs up to and including step i
     int* P;          // [nd][3][pcap] first step beyond r cells on axis b
     int* C;          // [nd][3][pcap] first run beyond r cells on axis b (not the run axis)
+    int* D;          // [nd][lcap] row-layout offset of step i's cell from the source's leaf (NULL: not kept)
+    void* ds;        // [nd][lcap] length of step i (float or double)
     int lcap, pcap;
 };
 
@@ -98,7 +100,8 @@ struct BeamTables {
 template <class T>
 struct RunTable {
     BeamRun<T>* run;
-    int *fb, *P, *C;
+    int *fb, *P, *C, *D;
+    T* ds;
     const WalkCounters* wc;
     int n, nr, k, cap, pcap, raxis;
     uint32_t prev;
@@ -139,7 +142,13 @@ struct RunTable {
             run[nr - 1].ds[k] = (T)d;
             run[nr - 1].k = k + 1;
         }
-        if (n < cap) fb[n] = (int)wc->exit_fb;
+        if (n < cap) {
+            fb[n] = (int)wc->exit_fb;
+            if (D) {
+                D[n] = off;
+                ds[n] = (T)d;
+            }
+        }
         k++;
         n++;
     }
@@ -225,6 +234,8 @@ __device__ __forceinline__ bool beam_table(const DevTree& t, const DirConst* __r
     rec.fb = tab.fb + (size_t)q * tab.lcap;
     rec.P = tab.P + (size_t)q * 3 * tab.pcap;
     rec.C = tab.C + (size_t)q * 3 * tab.pcap;
+    rec.D = tab.D ? tab.D + (size_t)q * tab.lcap : nullptr;
+    rec.ds = (T*)tab.ds + (size_t)q * tab.lcap;
     rec.wc = &wc;
     rec.n = rec.nr = rec.k = 0;
     rec.cap = tab.lcap;
@@ -426,6 +437,7 @@ struct BeamArgs {
     const void* field[2];   // row layouts along x and along y (adjoint: the slice, in either)
     const BeamRef* ref;
     const uint32_t* out;    // a bit per source: left out
+    unsigned long long* queue;  // units handed out so far
     int q0, nq, dgroup;     // directions [q0, q0 + nq), dgroup at a time
     long long blocks;       // 32^3-leaf blocks the sources can touch
 };
@@ -531,10 +543,91 @@ __host__ __device__ constexpr int beam_r()
 {
     return MODE == RT_MODE_FP64 ? (SM >= 4 ? 2 : 4) : (SM >= 8 ? 4 : 8);
 }
-template <int MODE, int SM>
+template <int MODE, int SM, int R>
 __host__ __device__ constexpr int beam_blocks()
 {
+    if (R == 1) return MODE == RT_MODE_FP64 ? (SM >= 8 ? 3 : SM >= 4 ? 4 : SM >= 2 ? 6 : 8) : (SM >= 8 ? 6 : 8);
+    if (MODE == RT_MODE_F32_KAHAN && SM == 4 && R == 4) return 5;
     return MODE == RT_MODE_FP64 ? (SM >= 8 ? 2 : 4) : (SM >= 8 ? 3 : 4);
+}
+
+// Leaves a thread takes in the adjoint.  It is launched one direction at a time,
+// so a launch has a twelfth (Nside 1) of the columns' units, and on a small cube
+// a long row leaves the chip short of warps: there a thread takes one leaf and
+// four steps' cells at once (add_steps).  Adjoint of a 64^3 cube, all directions,
+// us, one leaf against beam_r: F32-Kahan 1 species 293 / 437, 4 397 / 599, 8 650
+// / 719; FP64 472 / 702, 1240 / 1405, 2231 / 2368.  Of a 128^3 cube: F32-Kahan
+// 1497 / 1313, 2867 / 2844, 5431 / 4837; FP64 1 species 3931 / 4146, 2 7186 /
+// 7370, 4 13436 / 13268, 8 25758 / 26132 (more registers; at 256^3 FP64 1
+// species 51.0 / 50.6 ms).  F32-Kahan, 4 species: 4 leaves at 96 registers against
+// 8, 128^3 2760 / 2844, 256^3 27.9 / 26.0 ms.
+template <int MODE, int SM>
+__host__ __device__ constexpr int beam_adjoint_r(int level)
+{
+    return level <= (MODE == RT_MODE_FP64 && SM <= 2 ? 7 : 6) ? 1
+         : MODE == RT_MODE_F32_KAHAN && SM == 4 && level == 7 ? 4 : beam_r<MODE, SM>();
+}
+
+// The runs [0, nr) of a direction's n_run for R leaves in a row (ahead: cells of the cube from
+// the first leaf on, itself among them).  The next run's entry is read ahead of
+// its use.
+template <int MODE, int SM, int R, int OP, class T>
+__device__ __forceinline__ void add_runs(BeamSum<MODE, SM, OP> sum[R], const BeamRun<T>* __restrict__ run, int nr,
+                                         int n_run, int ahead, const T* __restrict__ base, long long rs)
+{
+    int4 h;
+    T ds[kRun];
+    load_run(run, h, ds);
+    for (int e = 0; e < nr; e++) {
+        int4 hn;
+        T dn[kRun];
+        load_run(run + min(e + 1, n_run - 1), hn, dn);
+        const int lim = ahead - h.y;
+        if (lim <= 0) break;
+        const T* p = base + (long long)(OP == kBeamAdjoint ? -h.x : h.x) * SM;
+        if (lim >= R + h.z - 1) {
+            switch (h.z) {
+            case 1: whole_run<MODE, SM, R, OP, 1>(sum, p, rs, ds); break;
+            case 2: whole_run<MODE, SM, R, OP, 2>(sum, p, rs, ds); break;
+            case 3: whole_run<MODE, SM, R, OP, 3>(sum, p, rs, ds); break;
+            default: whole_run<MODE, SM, R, OP, 4>(sum, p, rs, ds); break;
+            }
+        } else {
+            cut_run<MODE, SM, R, OP>(sum, p, rs, h.z, lim, ds);
+        }
+        h = hn;
+#pragma unroll
+        for (int k = 0; k < kRun; k++) ds[k] = dn[k];
+    }
+}
+
+// The steps [0, n) of direction q for one leaf of the adjoint, kSteps cells
+// loaded before the first is added: with one leaf a thread and few warps in
+// flight it is the wait for the cells that counts, and a run holds as few as one.
+constexpr int kSteps = 4;
+template <int MODE, int SM, int OP, class T>
+__device__ __forceinline__ void add_steps(BeamSum<MODE, SM, OP>& sum, const BeamTables& tab, int q, int n,
+                                          const T* __restrict__ base)
+{
+    const int* __restrict__ D = tab.D + (size_t)q * tab.lcap;
+    const T* __restrict__ ds = (const T*)tab.ds + (size_t)q * tab.lcap;
+    int i = 0;
+    for (; i + kSteps <= n; i += kSteps) {
+        const int4 at = __ldg((const int4*)(D + i));
+        T d[kSteps], v[kSteps][SM];
+        load_row<T, kSteps>(ds + i, d);
+        load_row<T, SM>(base - (long long)at.x * SM, v[0]);
+        load_row<T, SM>(base - (long long)at.y * SM, v[1]);
+        load_row<T, SM>(base - (long long)at.z * SM, v[2]);
+        load_row<T, SM>(base - (long long)at.w * SM, v[3]);
+#pragma unroll
+        for (int u = 0; u < kSteps; u++) sum.add(v[u], d[u]);
+    }
+    for (; i < n; i++) {
+        T v[SM];
+        load_row<T, SM>(base - (long long)__ldg(D + i) * SM, v);
+        sum.add(v, __ldg(ds + i));
+    }
 }
 
 // Units of a leaf block of edge B and one direction: R leaves a warp along the
@@ -552,7 +645,7 @@ __host__ __device__ __forceinline__ int beam_units(int B, int R, int W)
 // flight lie close together (their cells stay in L2) and a leaf's outputs for
 // dgroup directions are written close in time (they meet in L2).
 template <int MODE, int SM, int R, int OP>
-__global__ void __launch_bounds__(32 * kBeamWarps, beam_blocks<MODE, SM>()) k_beam(const BeamArgs a)
+__global__ void __launch_bounds__(32 * kBeamWarps, beam_blocks<MODE, SM, R>()) k_beam(const BeamArgs a)
 {
     using T = typename std::conditional<MODE == RT_MODE_FP64, double, float>::type;
     if (*(volatile const int*)&a.t.st->gather_off) return;
@@ -567,12 +660,16 @@ __global__ void __launch_bounds__(32 * kBeamWarps, beam_blocks<MODE, SM>()) k_be
     const uint32_t j0 = OP == kBeamAdjoint ? 0u : (uint32_t)a.ref->j0;
     const long long total = a.blocks * a.nq * U;
     unsigned long long n_segs = 0, n_rays = 0, n_efb = 0;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_unit = atomicAdd(&a.t.st->queue, 1ull);
-        __syncthreads();
-        const long long u = (long long)s_unit;
-        if (u >= total) break;
+    const bool once = R == 1 && total <= gridDim.x;  // a block a unit needs no queue (32^3, 1 species: 178 -> 166 us)
+    for (bool first_unit = true;; first_unit = false) {
+        long long u = blockIdx.x;
+        if (!once) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_unit = atomicAdd(a.queue, 1ull);
+            __syncthreads();
+            u = (long long)s_unit;
+        }
+        if (u >= total || (once && !first_unit)) break;
         const int ut = (int)(u % U);
         const long long v = u / U;
         const int qd = (int)(v % a.dgroup);
@@ -617,34 +714,13 @@ __global__ void __launch_bounds__(32 * kBeamWarps, beam_blocks<MODE, SM>()) k_be
         const int ahead = upR ? N - first : first + 1;  // itself among them
         const long long rs = (long long)(upR ? st_r : -st_r) * SM;
         const T* __restrict__ base = (const T*)a.field[ax.lane] + ((long long)cl + (long long)ct * st_t + (long long)first * st_r) * SM;
-        const BeamRun<T>* __restrict__ run = (const BeamRun<T>*)a.tab.run + (size_t)q * a.tab.lcap;
         BeamSum<MODE, SM, OP> sum[R];  // sum[r]: leaf `first` + r steps forward
 #pragma unroll
         for (int r = 0; r < R; r++) sum[r].init();
-        int4 h;
-        T ds[kRun];
-        load_run(run, h, ds);
-        for (int e = 0; e < nr; e++) {
-            int4 hn;
-            T dn[kRun];
-            load_run(run + min(e + 1, info.x - 1), hn, dn);  // the next run's entry, ahead of its use
-            const int lim = ahead - h.y;
-            if (lim <= 0) break;
-            const T* p = base + (long long)(OP == kBeamAdjoint ? -h.x : h.x) * SM;
-            if (lim >= R + h.z - 1) {
-                switch (h.z) {
-                case 1: whole_run<MODE, SM, R, OP, 1>(sum, p, rs, ds); break;
-                case 2: whole_run<MODE, SM, R, OP, 2>(sum, p, rs, ds); break;
-                case 3: whole_run<MODE, SM, R, OP, 3>(sum, p, rs, ds); break;
-                default: whole_run<MODE, SM, R, OP, 4>(sum, p, rs, ds); break;
-                }
-            } else {
-                cut_run<MODE, SM, R, OP>(sum, p, rs, h.z, lim, ds);
-            }
-            h = hn;
-#pragma unroll
-            for (int k = 0; k < kRun; k++) ds[k] = dn[k];
-        }
+        if constexpr (R == 1)
+            add_steps(sum[0], a.tab, q, min(steps, __ldg(Pq + ax.run * a.tab.pcap + ahead - 1)), base);
+        else
+            add_runs<MODE, SM, R, OP>(sum, (const BeamRun<T>*)a.tab.run + (size_t)q * a.tab.lcap, nr, info.x, ahead, base, rs);
 #pragma unroll
         for (int r = 0; r < R; r++) {
             const int c = upR ? first + r : first - r;
@@ -690,10 +766,35 @@ __global__ void __launch_bounds__(32 * kBeamWarps, beam_blocks<MODE, SM>()) k_be
             }
         }
     }
-    __syncwarp();
-    flush_counters(a.t.st, n_rays, n_segs, n_efb, 0ull);
+    if constexpr (R > 1) {
+        __syncwarp();
+        flush_counters(a.t.st, n_rays, n_segs, n_efb, 0ull);
+    } else {
+        // the adjoint of a small cube is a launch of some microseconds a direction, and
+        // additions to one address follow one another at about 2 ns each: one a
+        // block and not one a warp (64^3, 1 species, 309 -> 293 us)
+        __shared__ unsigned long long s_sum[2];
+        __syncthreads();
+        if (threadIdx.x < 2) s_sum[threadIdx.x] = 0ull;
+        __syncthreads();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            n_rays += __shfl_down_sync(RT_FULL, n_rays, o);
+            n_segs += __shfl_down_sync(RT_FULL, n_segs, o);
+        }
+        if (lane == 0) {
+            atomicAdd(s_sum, n_rays);
+            atomicAdd(s_sum + 1, n_segs);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && s_sum[0]) {
+            atomicAdd(&a.t.st->rays, s_sum[0]);
+            atomicAdd(&a.t.st->segments, s_sum[1]);
+        }
+    }
 }
 
+// Launches k_beam for the directions [g.q0, g.q0 + g.nq), units handed out over g.queue.
 template <int MODE, int SM, int R, int OP>
 static cudaError_t go_beam(const BeamArgs& g, cudaStream_t s)
 {
@@ -704,9 +805,25 @@ static cudaError_t go_beam(const BeamArgs& g, cudaStream_t s)
     const int B = std::min(32, 1 << g.t.t.uniform_level);
     const long long units = g.blocks * g.nq * beam_units(B, R, W);
     const int grid = (int)std::min<long long>(units, (long long)sm_count_of(dev) * std::max(1, fit));
-    cudaMemsetAsync(&g.t.st->queue, 0, sizeof(unsigned long long), s);
-    k_beam<MODE, SM, R, OP><<<grid, 32 * W, 0, s>>>(g);
-    return cudaGetLastError();
+    if (cudaMemsetAsync(g.queue, 0, sizeof(unsigned long long) * (OP == kBeamAdjoint ? g.t.nd : 1), s) != cudaSuccess)
+        return cudaGetLastError();
+    if (OP != kBeamAdjoint) {
+        k_beam<MODE, SM, R, OP><<<grid, 32 * W, 0, s>>>(g);
+        return cudaGetLastError();
+    }
+    // one direction after another
+    using T = typename std::conditional<MODE == RT_MODE_FP64, double, float>::type;
+    const int sgrid = (int)std::min<long long>((g.t.n_src + 255) / 256, (long long)sm_count_of(dev) * 16);
+    BeamArgs d = g;
+    for (int q = 0; q < g.t.nd; q++) {
+        k_beam_slice<T, SM><<<sgrid, 256, 0, s>>>((const T*)g.t.gin, g.t.dirs, q, g.t.nd, g.t.t.uniform_level, (T*)g.field[0], g.t.st);
+        d.q0 = q;
+        d.queue = g.queue + q;
+        k_beam<MODE, SM, R, OP><<<grid, 32 * W, 0, s>>>(d);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 template <int MODE, int SM>
@@ -714,7 +831,10 @@ static cudaError_t go_beam_op(const BeamArgs& g, int op, cudaStream_t s)
 {
     constexpr int R = beam_r<MODE, SM>();
     if (op == kBeamAdjoint) {
-        if (g.t.t.uniform_level < 3) return go_beam<MODE, SM, 1, kBeamAdjoint>(g, s);
+        const int r = beam_adjoint_r<MODE, SM>(g.t.t.uniform_level);
+        if (r == 1) return go_beam<MODE, SM, 1, kBeamAdjoint>(g, s);
+        if constexpr (beam_adjoint_r<MODE, SM>(7) == 4 && R != 4)
+            if (r == 4) return go_beam<MODE, SM, 4, kBeamAdjoint>(g, s);
         return go_beam<MODE, SM, R, kBeamAdjoint>(g, s);
     }
     if (op == kBeamEpilogue) return go_beam<MODE, SM, R, kBeamEpilogue>(g, s);
@@ -733,20 +853,24 @@ struct BeamScratch {
     BeamTables tab;
     BeamRef* ref;
     uint32_t *out, *rest;
+    unsigned long long* queue;
     unsigned int most;
 };
 
-static size_t beam_scratch(char* p, int nd, int L, int64_t n_src, int mode, BeamScratch* b)
+static size_t beam_scratch(char* p, int nd, int L, int64_t n_src, int mode, bool adjoint, BeamScratch* b)
 {
     const int N = 1 << L;
     const int lcap = (3 * N + 3 + 15) / 16 * 16, pcap = (N + 1 + 3) / 4 * 4;
     const size_t rsz = mode == RT_MODE_FP64 ? sizeof(BeamRun<double>) : sizeof(BeamRun<float>);
     const unsigned int most = (unsigned int)(n_src / 16);
+    const size_t steps = adjoint ? (size_t)nd * lcap : 0;
+    // the tables first, at places that do not depend on n_src: a later call finds them there
     const size_t bytes[] = {sizeof(BeamRef), (size_t)nd * sizeof(int4), (size_t)nd * lcap * rsz, (size_t)nd * lcap * 4,
-                            (size_t)nd * 3 * pcap * 4, (size_t)nd * 3 * pcap * 4, (size_t)((n_src + 31) / 32) * 4,
-                            (size_t)most * 4};
-    size_t at[9] = {0};
-    for (int i = 0; i < 8; i++) at[i + 1] = at[i] + round256(bytes[i]);
+                            (size_t)nd * 3 * pcap * 4, (size_t)nd * 3 * pcap * 4, steps * 4,
+                            steps * (mode == RT_MODE_FP64 ? 8 : 4), (size_t)(adjoint ? nd : 1) * 8,
+                            (size_t)((n_src + 31) / 32) * 4, (size_t)most * 4};
+    size_t at[12] = {0};
+    for (int i = 0; i < 11; i++) at[i + 1] = at[i] + round256(bytes[i]);
     if (p) {
         b->ref = (BeamRef*)(p + at[0]);
         b->tab.info = (int4*)(p + at[1]);
@@ -754,13 +878,16 @@ static size_t beam_scratch(char* p, int nd, int L, int64_t n_src, int mode, Beam
         b->tab.fb = (int*)(p + at[3]);
         b->tab.P = (int*)(p + at[4]);
         b->tab.C = (int*)(p + at[5]);
-        b->out = (uint32_t*)(p + at[6]);
-        b->rest = (uint32_t*)(p + at[7]);
+        b->tab.D = adjoint ? (int*)(p + at[6]) : nullptr;
+        b->tab.ds = adjoint ? p + at[7] : nullptr;
+        b->queue = (unsigned long long*)(p + at[8]);
+        b->out = (uint32_t*)(p + at[9]);
+        b->rest = (uint32_t*)(p + at[10]);
         b->tab.lcap = lcap;
         b->tab.pcap = pcap;
         b->most = most;
     }
-    return at[8];
+    return at[11];
 }
 
 // Enqueues the source check (most: sources that may be left out) and the tables.
@@ -788,19 +915,6 @@ bool gather_applies(const rt_octree* t, const TraceArgs& a)
            (a.S == 1 || a.S == 2 || a.S == 4 || a.S == 8);
 }
 
-template <int MODE, int SM>
-static cudaError_t go_gather(BeamArgs g, void* gl, int sgrid, cudaStream_t s)
-{
-    using T = typename std::conditional<MODE == RT_MODE_FP64, double, float>::type;
-    for (int q = 0; q < g.t.nd; q++) {
-        k_beam_slice<T, SM><<<sgrid, 256, 0, s>>>((const T*)g.t.gin, g.t.dirs, q, g.t.nd, g.t.t.uniform_level, (T*)gl, g.t.st);
-        g.q0 = q;
-        const cudaError_t e = go_beam_op<MODE, SM>(g, kBeamAdjoint, s);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 // Enqueues the source check, the tables and the gather on `s`: one direction
 // after another (the stream orders them, so each leaf's gradient takes its
 // directions in a fixed order and no two threads update it at once).  The
@@ -808,7 +922,7 @@ static cudaError_t go_gather(BeamArgs g, void* gl, int sgrid, cudaStream_t s)
 int launch_adjoint_gather(rt_octree* t, const TraceArgs& a, int mode, cudaStream_t s)
 {
     const size_t tsz = mode == RT_MODE_FP64 ? 8 : 4;
-    const size_t t_bytes = beam_scratch(nullptr, a.nd, a.t.uniform_level, a.n_src, mode, nullptr);
+    const size_t t_bytes = beam_scratch(nullptr, a.nd, a.t.uniform_level, a.n_src, mode, true, nullptr);
     const size_t need = t_bytes + (size_t)a.n_src * a.S * tsz;
     if (t->adj_tab_bytes < need) {
         if (t->adj_tab) {
@@ -828,24 +942,22 @@ int launch_adjoint_gather(rt_octree* t, const TraceArgs& a, int mode, cudaStream
     memset(&g, 0, sizeof g);
     g.t = a;
     BeamScratch b;
-    beam_scratch((char*)t->adj_tab, a.nd, a.t.uniform_level, a.n_src, mode, &b);
+    beam_scratch((char*)t->adj_tab, a.nd, a.t.uniform_level, a.n_src, mode, true, &b);
     g.tab = b.tab;
+    g.queue = b.queue;
     char* gl = (char*)t->adj_tab + t_bytes;
     g.field[0] = g.field[1] = gl;
     g.nq = g.dgroup = 1;
     const int L = a.t.uniform_level;
     g.blocks = L >= 5 ? 1ll << (3 * (L - 5)) : 1;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const int sgrid = (int)std::min<long long>((a.n_src + 255) / 256, (long long)sm_count_of(dev) * 16);
     cudaError_t e = beam_setup(a, mode, b, 0, s);  // a source left out: no gather
     if (e == cudaSuccess) {
         if (mode == RT_MODE_FP64)
-            e = a.S == 1 ? go_gather<RT_MODE_FP64, 1>(g, gl, sgrid, s) : a.S == 2 ? go_gather<RT_MODE_FP64, 2>(g, gl, sgrid, s)
-              : a.S == 4 ? go_gather<RT_MODE_FP64, 4>(g, gl, sgrid, s) : go_gather<RT_MODE_FP64, 8>(g, gl, sgrid, s);
+            e = a.S == 1 ? go_beam_op<RT_MODE_FP64, 1>(g, kBeamAdjoint, s) : a.S == 2 ? go_beam_op<RT_MODE_FP64, 2>(g, kBeamAdjoint, s)
+              : a.S == 4 ? go_beam_op<RT_MODE_FP64, 4>(g, kBeamAdjoint, s) : go_beam_op<RT_MODE_FP64, 8>(g, kBeamAdjoint, s);
         else
-            e = a.S == 1 ? go_gather<RT_MODE_F32_KAHAN, 1>(g, gl, sgrid, s) : a.S == 2 ? go_gather<RT_MODE_F32_KAHAN, 2>(g, gl, sgrid, s)
-              : a.S == 4 ? go_gather<RT_MODE_F32_KAHAN, 4>(g, gl, sgrid, s) : go_gather<RT_MODE_F32_KAHAN, 8>(g, gl, sgrid, s);
+            e = a.S == 1 ? go_beam_op<RT_MODE_F32_KAHAN, 1>(g, kBeamAdjoint, s) : a.S == 2 ? go_beam_op<RT_MODE_F32_KAHAN, 2>(g, kBeamAdjoint, s)
+              : a.S == 4 ? go_beam_op<RT_MODE_F32_KAHAN, 4>(g, kBeamAdjoint, s) : go_beam_op<RT_MODE_F32_KAHAN, 8>(g, kBeamAdjoint, s);
     }
     if (e != cudaSuccess) return cuda_error("rt_trace_columns_adjoint: gather launch");
     return RT_OK;
@@ -860,7 +972,7 @@ size_t beam_bytes(const rt_octree* t, int64_t n_src, int nd, int S, int mode)
 {
     const int L = t->uniform_allowed ? t->dev.uniform_level : -1;
     if (L < 5 || n_src < 32 || n_src > t->dev.n || n_src * 16 < t->dev.n || t->dev.step_cap < t->default_cap) return 0;
-    const size_t tab = beam_scratch(nullptr, nd, L, n_src, mode, nullptr);
+    const size_t tab = beam_scratch(nullptr, nd, L, n_src, mode, false, nullptr);
     if (tab > (256ull << 20) + (size_t)n_src / 2) return 0;
     return tab + 2 * round256((size_t)t->dev.n * padded_species(S) * (mode == RT_MODE_FP64 ? 8 : 4));
 }
@@ -911,14 +1023,15 @@ int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check,
         cudaMemsetAsync(t->fwd_tab, 0, sizeof(BeamRef), s);  // no tables yet
     }
     const int L = a.t.uniform_level, SM = padded_species(a.S);
-    const size_t t_bytes = beam_scratch(nullptr, a.nd, L, a.n_src, mode, nullptr);
+    const size_t t_bytes = beam_scratch(nullptr, a.nd, L, a.n_src, mode, false, nullptr);
     const size_t row_bytes = round256((size_t)t->dev.n * SM * (mode == RT_MODE_FP64 ? 8 : 4));
     BeamArgs g;
     memset(&g, 0, sizeof g);
     g.t = a;
     BeamScratch b;
-    beam_scratch((char*)t->fwd_tab, a.nd, L, a.n_src, mode, &b);
+    beam_scratch((char*)t->fwd_tab, a.nd, L, a.n_src, mode, false, &b);
     g.tab = b.tab;
+    g.queue = b.queue;
     g.ref = b.ref;
     g.out = b.out;
     void* rows[2] = {(char*)t->fwd_tab + t_bytes, (char*)t->fwd_tab + t_bytes + row_bytes};

@@ -92,6 +92,34 @@ def test_gather_matches_oracle(rt, level, S, nside):
     tree.close()
 
 
+@pytest.mark.parametrize("level,S", [(0, 1), (0, 8), (1, 2), (2, 8), (3, 4), (4, 2), (5, 1), (5, 2), (5, 8), (6, 2), (6, 4), (6, 8),
+                                     (7, 1), (7, 2), (7, 4), (7, 8)])
+@pytest.mark.parametrize("mode", ["fp64", "f32k"])
+def test_gather_matches_scatter(rt, level, S, mode):
+    """Every number of leaves a thread takes (one on small cubes, more on larger
+    ones) and every species count, against the scatter, which adds the products
+    of the same lengths in FP64.  FP64: two sums of the same terms, each within
+    a rounding a term (at most 24 N of them, 3e-13 at 128^3).  F32-Kahan: each
+    product rounds to FP32 once and a Kahan sum is within two roundings of the
+    magnitudes, 3 * 2^-24 in all; the scatter's products are exact."""
+    import torch
+    keys, lev = uniform_octree(level)
+    tree = rt.Octree(_dev(keys), _dev(lev))
+    src = _dev(_centres(keys, lev))
+    gen = torch.Generator(device="cuda").manual_seed(1000 + 10 * level + S)
+    g = torch.randn((keys.shape[0], 12, S), generator=gen, device="cuda",
+                    dtype=torch.float64 if mode == "fp64" else torch.float32)
+    got, st = _run(rt, tree, src, 1, g, mode)
+    sc, st_sc = _run(rt, tree, src, 1, g, mode, policy=1)
+    mag, _ = _run(rt, tree, src, 1, g.abs(), mode, policy=1)
+    assert st["gathered"] == 1 and st_sc["gathered"] == 0
+    assert (st["rays"], st["segments"]) == (st_sc["rays"], st_sc["segments"])
+    _bound_check(got, sc, mag, 1e-12 if mode == "fp64" else 4 * 2.0 ** -24)
+    again, _ = _run(rt, tree, src, 1, g, mode)
+    assert np.array_equal(got.view(np.uint64), again.view(np.uint64))
+    tree.close()
+
+
 @pytest.mark.parametrize("fine", [0, 1])
 def test_gather_common_offset_not_centre(rt, fine):
     """Every source at the same off-centre offset in its leaf, on the depth-21
