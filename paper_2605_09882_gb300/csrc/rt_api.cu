@@ -327,7 +327,7 @@ int rt::trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_sr
     if (a.pair) a.n_src_pad = (n_src + 63) / 64 * 64;
     const int fit = a.pair ? occupancy_pair(n_species, g_block)
                            : occupancy_fwd(0, mode, n_species, a.t.uniform_level >= 0, g_block);
-    if (cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
+    if (!beam && cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
         return cuda_error("rt_trace_columns: queue reset");
     const int grid = grid_for(fit);
     spread_rays(a, (long long)grid * (g_block / 32));

@@ -168,13 +168,16 @@ struct BeamRef {
 };
 
 // One warp: the most common offset (and leaf minus index) among 32 sources
-// spread over the list, and the reset of the check's results.  The tables
+// spread over the list, and the reset of the check's results and of the queues.
+// Fewer than `need` of the 32 at that offset settle it: st->gather_off is set
+// and nothing more is prepared for a form that cannot apply (scattered points).
+// The tables
 // depend on the level, the mode, the directions and the offset alone: those of
 // an earlier call on this scratch with the same values stand (a walk of a few
 // hundred steps by one thread a direction: 26 us at 32^3, 48 us at 128^3, which
 // a trace in source chunks would pay for each chunk).
-__global__ void k_beam_ref(const double* __restrict__ src, long long n, int L, unsigned int key, int nd, BeamRef* ref,
-                           DevStats* st)
+__global__ void k_beam_ref(const double* __restrict__ src, long long n, int L, unsigned int key, int nd, int need,
+                           BeamRef* ref, unsigned long long* queue, int queues, DevStats* st)
 {
     const int lane = threadIdx.x;
     const long long s = (n - 1) * lane / 31;
@@ -198,7 +201,9 @@ __global__ void k_beam_ref(const double* __restrict__ src, long long n, int L, u
     }
     const int most = __reduce_max_sync(RT_FULL, votes);
     const unsigned who = __ballot_sync(RT_FULL, votes == most);
+    for (int i = lane; i < queues; i += 32) queue[i] = 0ull;
     if (lane == __ffs(who) - 1) {
+        st->queue = 0ull;  // the walk's, launched after this form
         if (ref->key != key || ref->done != (unsigned int)nd || ref->f[0] != f[0] || ref->f[1] != f[1] || ref->f[2] != f[2]) {
             ref->key = key;
             ref->done = 0u;
@@ -210,7 +215,7 @@ __global__ void k_beam_ref(const double* __restrict__ src, long long n, int L, u
         }
         ref->j0 = j0;
         ref->n_rest = 0u;
-        st->gather_off = (j0 < 0 || j0 + n > (1ll << (3 * L))) ? 1 : 0;
+        st->gather_off = (votes < need || j0 < 0 || j0 + n > (1ll << (3 * L))) ? 1 : 0;
     }
 }
 
@@ -376,37 +381,44 @@ __device__ __forceinline__ uint32_t row_leaf(unsigned long long i, int L, int la
     return spread10(x) | (spread10(y) << 1) | (spread10(z) << 2);
 }
 
-// The densities in row layout, SM values a leaf (zeros past S), in the type
-// the columns are summed in (the conversion the walk makes on each load).
-// With check, each density is checked as k_check_dens does; that part runs
-// whether or not the sources have the shared offset.
+// The densities of leaf j, SM values (zeros past S), in the type the columns are
+// summed in (the conversion the walk makes on each load); with check, checked as
+// k_check_dens does.
 template <class T, int SM>
-__global__ void k_beam_dens(const void* __restrict__ dens, int f64, int S, int L, int lane, T* __restrict__ out,
-                            int check, DevStats* st)
+__device__ __forceinline__ void beam_dens(const void* __restrict__ dens, int f64, int S, uint32_t j, T v[SM], bool check,
+                                          DevStats* st)
+{
+    if (S == SM && !f64) load_dens<SM, T>(dens, 0, SM, j, v);
+    else load_dens<SM, T>(dens, f64, S, j, v);
+    if (!check) return;
+    bool bad = false;
+    if (f64) {
+        for (int k = 0; k < S; k++) {
+            const double w = __ldg((const double*)dens + (size_t)j * S + k);
+            bad |= !(w >= 0.0 && w <= 1.7976931348623157e308);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < SM; k++) bad |= !(v[k] >= (T)0 && v[k] <= (T)3.402823466e38f);
+    }
+    if (bad) report_fault(st, RT_ERR_NONFINITE, (long long)j);
+}
+
+// The densities in row layout along x, then along y.  The check runs whether or
+// not the sources have the shared offset.
+template <class T, int SM>
+__global__ void k_beam_dens(const void* __restrict__ dens, int f64, int S, int L, T* __restrict__ along_x,
+                            T* __restrict__ along_y, int check, DevStats* st)
 {
     const bool off = *(volatile const int*)&st->gather_off != 0;
-    if (off && !check) return;
-    const unsigned long long n = 1ull << (3 * L);
-    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
+    const unsigned long long n = 1ull << (3 * L), end = off ? (check ? n : 0ull) : 2ull * n;
+    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < end;
          i += (unsigned long long)gridDim.x * blockDim.x) {
-        const uint32_t j = row_leaf(i, L, lane);
+        const bool y = i >= n;
+        const unsigned long long r = y ? i - n : i;
         T v[SM];
-        if (S == SM && !f64) load_dens<SM, T>(dens, 0, SM, j, v);
-        else load_dens<SM, T>(dens, f64, S, j, v);
-        if (check) {
-            bool bad = false;
-            if (f64) {
-                for (int k = 0; k < S; k++) {
-                    const double w = __ldg((const double*)dens + (size_t)j * S + k);
-                    bad |= !(w >= 0.0 && w <= 1.7976931348623157e308);
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < SM; k++) bad |= !(v[k] >= (T)0 && v[k] <= (T)3.402823466e38f);
-            }
-            if (bad) report_fault(st, RT_ERR_NONFINITE, (long long)j);
-        }
-        if (!off) store_row<T, SM>(out + (size_t)i * SM, v);
+        beam_dens<T, SM>(dens, f64, S, off ? (uint32_t)r : row_leaf(r, L, y), v, check && !y, st);
+        if (!off) store_row<T, SM>((y ? along_y : along_x) + (size_t)r * SM, v);
     }
 }
 
@@ -437,7 +449,7 @@ struct BeamArgs {
     const void* field[2];   // row layouts along x and along y (adjoint: the slice, in either)
     const BeamRef* ref;
     const uint32_t* out;    // a bit per source: left out
-    unsigned long long* queue;  // units handed out so far
+    unsigned long long* queue;  // units handed out so far (adjoint: one a direction)
     int q0, nq, dgroup;     // directions [q0, q0 + nq), dgroup at a time
     long long blocks;       // 32^3-leaf blocks the sources can touch
 };
@@ -805,8 +817,6 @@ static cudaError_t go_beam(const BeamArgs& g, cudaStream_t s)
     const int B = std::min(32, 1 << g.t.t.uniform_level);
     const long long units = g.blocks * g.nq * beam_units(B, R, W);
     const int grid = (int)std::min<long long>(units, (long long)sm_count_of(dev) * std::max(1, fit));
-    if (cudaMemsetAsync(g.queue, 0, sizeof(unsigned long long) * (OP == kBeamAdjoint ? g.t.nd : 1), s) != cudaSuccess)
-        return cudaGetLastError();
     if (OP != kBeamAdjoint) {
         k_beam<MODE, SM, R, OP><<<grid, 32 * W, 0, s>>>(g);
         return cudaGetLastError();
@@ -867,7 +877,7 @@ static size_t beam_scratch(char* p, int nd, int L, int64_t n_src, int mode, bool
     // the tables first, at places that do not depend on n_src: a later call finds them there
     const size_t bytes[] = {sizeof(BeamRef), (size_t)nd * sizeof(int4), (size_t)nd * lcap * rsz, (size_t)nd * lcap * 4,
                             (size_t)nd * 3 * pcap * 4, (size_t)nd * 3 * pcap * 4, steps * 4,
-                            steps * (mode == RT_MODE_FP64 ? 8 : 4), (size_t)(adjoint ? nd : 1) * 8,
+                            steps * (mode == RT_MODE_FP64 ? 8 : 4), (size_t)(adjoint ? nd : 2) * 8,
                             (size_t)((n_src + 31) / 32) * 4, (size_t)most * 4};
     size_t at[12] = {0};
     for (int i = 0; i < 11; i++) at[i + 1] = at[i] + round256(bytes[i]);
@@ -890,14 +900,21 @@ static size_t beam_scratch(char* p, int nd, int L, int64_t n_src, int mode, bool
     return at[11];
 }
 
-// Enqueues the source check (most: sources that may be left out) and the tables.
-static cudaError_t beam_setup(const TraceArgs& a, int mode, const BeamScratch& b, unsigned int most, cudaStream_t s)
+// Sources of 32 at the commonest offset below which a form that may leave out a
+// sixteenth is not tried.  With a sixteenth elsewhere at random, fewer than 24
+// agree once in 9,000 calls (and the walk then does what the form would have);
+// with half elsewhere, more than 23 once in 280.
+constexpr int kBeamVotes = 24;
+
+// Enqueues the source check (most: sources that may be left out) and the tables,
+// and resets the queues.
+static cudaError_t beam_setup(const TraceArgs& a, int mode, const BeamScratch& b, unsigned int most, int queues, cudaStream_t s)
 {
     int dev = 0;
     cudaGetDevice(&dev);
     const int grid = a.nd + (int)std::max<long long>(1, std::min<long long>((a.n_src + 255) / 256, (long long)sm_count_of(dev) * 8));
     const unsigned int key = 1u | (unsigned)a.t.uniform_level << 1 | (unsigned)mode << 6 | (unsigned)a.nd << 7;
-    k_beam_ref<<<1, 32, 0, s>>>(a.src, a.n_src, a.t.uniform_level, key, a.nd, b.ref, a.st);
+    k_beam_ref<<<1, 32, 0, s>>>(a.src, a.n_src, a.t.uniform_level, key, a.nd, most ? kBeamVotes : 32, b.ref, b.queue, queues, a.st);
     if (mode == RT_MODE_FP64)
         k_beam_setup<RT_MODE_FP64><<<grid, 256, 0, s>>>(a.t, a.dirs, a.nd, a.src, a.n_src, b.ref, b.tab, b.out, b.rest, most, a.st);
     else
@@ -950,7 +967,7 @@ int launch_adjoint_gather(rt_octree* t, const TraceArgs& a, int mode, cudaStream
     g.nq = g.dgroup = 1;
     const int L = a.t.uniform_level;
     g.blocks = L >= 5 ? 1ll << (3 * (L - 5)) : 1;
-    cudaError_t e = beam_setup(a, mode, b, 0, s);  // a source left out: no gather
+    cudaError_t e = beam_setup(a, mode, b, 0, a.nd, s);  // a source left out: no gather
     if (e == cudaSuccess) {
         if (mode == RT_MODE_FP64)
             e = a.S == 1 ? go_beam_op<RT_MODE_FP64, 1>(g, kBeamAdjoint, s) : a.S == 2 ? go_beam_op<RT_MODE_FP64, 2>(g, kBeamAdjoint, s)
@@ -984,17 +1001,15 @@ static cudaError_t go_trace(const BeamArgs& g, void* const rows[2], bool check, 
     int dev = 0;
     cudaGetDevice(&dev);
     const int L = g.t.t.uniform_level;
-    const int grid = (int)std::min<long long>(1ll << (3 * L - 8), (long long)sm_count_of(dev) * 16);
-    for (int lane = 0; lane < 2; lane++)
-        k_beam_dens<T, SM><<<grid, 256, 0, s>>>(g.t.dens, g.t.dens_f64, g.t.S, L, lane, (T*)rows[lane],
-                                                check && lane == 0, g.t.st);
+    const int grid = (int)std::min<long long>(1ll << (3 * L - 7), (long long)sm_count_of(dev) * 16);
+    k_beam_dens<T, SM><<<grid, 256, 0, s>>>(g.t.dens, g.t.dens_f64, g.t.S, L, (T*)rows[0], (T*)rows[1], check, g.t.st);
     return go_beam_op<MODE, SM>(g, op, s);
 }
 
 // Enqueues the shared-offset forward trace (with the density check) or
 // epilogue on `s`, if the call's shape admits it; ran tells whether it did.
 // It sets a's gate and list of left-out sources for the walk launched after
-// it.  Its scratch belongs to the handle: a captured stream, or no memory for it, leaves the
+// it, and resets that walk's queue.  Its scratch belongs to the handle: a captured stream, or no memory for it, leaves the
 // call to the walk.
 int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check, cudaStream_t s, bool* ran)
 {
@@ -1041,7 +1056,7 @@ int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check,
     g.dgroup = a.dgroup > 1 ? a.dgroup : 1;
     g.blocks = std::min<long long>(1ll << (3 * (L - 5)), (a.n_src + 32767) / 32768 + 1);
     const int op = epilogue ? kBeamEpilogue : kBeamColumns;
-    cudaError_t e = beam_setup(a, mode, b, b.most, s);
+    cudaError_t e = beam_setup(a, mode, b, b.most, 2, s);
     if (e == cudaSuccess) {
         if (mode == RT_MODE_FP64)
             e = SM == 1 ? go_trace<RT_MODE_FP64, 1>(g, rows, check, op, s) : SM == 2 ? go_trace<RT_MODE_FP64, 2>(g, rows, check, op, s)
@@ -1054,6 +1069,7 @@ int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check,
     a.gate = &t->st->gather_off;
     a.rest = b.rest;
     a.n_rest = &b.ref->n_rest;
+    a.rest_queue = b.queue + 1;
     *ran = true;
     return RT_OK;
 }

@@ -5,18 +5,21 @@
 
 namespace rt {
 
-template <int MODE, bool U>
+template <int MODE, bool U, bool GATED = false>
 static cudaError_t go(const TraceArgs& a, int block, int grid, cudaStream_t s)
 {
-    if (a.S <= 1) k_trace<4, MODE, U, 1><<<grid, block, 0, s>>>(a);
-    else if (a.S <= 2) k_trace<4, MODE, U, 2><<<grid, block, 0, s>>>(a);
-    else if (a.S <= 4) k_trace<4, MODE, U, 4><<<grid, block, 0, s>>>(a);
-    else k_trace<4, MODE, U, 8><<<grid, block, 0, s>>>(a);
+    if (a.S <= 1) k_trace<4, MODE, U, 1, GATED><<<grid, block, 0, s>>>(a);
+    else if (a.S <= 2) k_trace<4, MODE, U, 2, GATED><<<grid, block, 0, s>>>(a);
+    else if (a.S <= 4) k_trace<4, MODE, U, 4, GATED><<<grid, block, 0, s>>>(a);
+    else k_trace<4, MODE, U, 8, GATED><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_epilogue(const TraceArgs& a, int mode, int block, int grid, cudaStream_t s)
 {
+    if (a.gate)
+        return mode == RT_MODE_FP64 ? go<RT_MODE_FP64, true, true>(a, block, grid, s)
+                                    : go<RT_MODE_F32_KAHAN, true, true>(a, block, grid, s);
     const bool u = a.t.uniform_level >= 0;
     if (mode == RT_MODE_FP64) return u ? go<RT_MODE_FP64, true>(a, block, grid, s) : go<RT_MODE_FP64, false>(a, block, grid, s);
     return u ? go<RT_MODE_F32_KAHAN, true>(a, block, grid, s) : go<RT_MODE_F32_KAHAN, false>(a, block, grid, s);
@@ -96,7 +99,7 @@ extern "C" int rt_trace_epilogue(const rt_octree* t, const double* d_src, int64_
     const int fit = occupancy_epi(mode, n_species, a.t.uniform_level >= 0, block);
     const int grid = sm_count_of(dev) * std::max(1, bps > 0 ? std::min(bps, fit) : fit);
     spread_rays(a, (long long)grid * (block / 32));
-    if (cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess ||
+    if ((!beam && cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess) ||
         launch_epilogue(a, mode, block, grid, s) != cudaSuccess)
         return cuda_error("rt_trace_epilogue: launch");
     if (h_epi->kind != RT_EPI_ATTENUATION) {

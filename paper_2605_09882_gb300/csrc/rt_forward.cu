@@ -3,17 +3,17 @@
 
 namespace rt {
 
-template <int KIND, int MODE, bool U>
+template <int KIND, int MODE, bool U, bool GATED = false>
 static cudaError_t go(const TraceArgs& a, int block, int grid, cudaStream_t s)
 {
     if (KIND == 1) {
         k_trace<1, MODE, U, 1><<<grid, block, 0, s>>>(a);
         return cudaGetLastError();
     }
-    if (a.S <= 1) k_trace<KIND, MODE, U, 1><<<grid, block, 0, s>>>(a);
-    else if (a.S <= 2) k_trace<KIND, MODE, U, 2><<<grid, block, 0, s>>>(a);
-    else if (a.S <= 4) k_trace<KIND, MODE, U, 4><<<grid, block, 0, s>>>(a);
-    else k_trace<KIND, MODE, U, 8><<<grid, block, 0, s>>>(a);
+    if (a.S <= 1) k_trace<KIND, MODE, U, 1, GATED><<<grid, block, 0, s>>>(a);
+    else if (a.S <= 2) k_trace<KIND, MODE, U, 2, GATED><<<grid, block, 0, s>>>(a);
+    else if (a.S <= 4) k_trace<KIND, MODE, U, 4, GATED><<<grid, block, 0, s>>>(a);
+    else k_trace<KIND, MODE, U, 8, GATED><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -37,9 +37,11 @@ cudaError_t launch_forward(const TraceArgs& a, int mode, int block, int grid, cu
         case 8: k_trace_pair<8><<<grid, block, 0, s>>>(a); break;
         default: return cudaErrorInvalidValue;
         }
-        if (!a.gate) return cudaGetLastError();
-        // then the sources the shared-offset form left out, one ray per lane
+        return cudaGetLastError();
     }
+    if (a.gate)
+        return mode == RT_MODE_FP64 ? go<0, RT_MODE_FP64, true, true>(a, block, grid, s)
+                                    : go<0, RT_MODE_F32_KAHAN, true, true>(a, block, grid, s);
     return dispatch<0>(a, mode, block, grid, s);
 }
 

@@ -83,8 +83,7 @@ struct TraceArgs {
     int gw;                  // rays a group: 32, or fewer to spread a call of few rays over the warps
     int layout;              // ray order: 0 direction-major (sources padded to 32), 1 source-major
     int dgroup;              // layout 0: directions per group (a power of two dividing nd; <= 1: one)
-    int pair;                // forward on a uniform cube: two rays per lane (k_trace_pair; n_src_pad % 64 == 0),
-                             // k_trace then only for the sources the shared-offset form left out
+    int pair;                // forward on a uniform cube: two rays per lane (k_trace_pair; n_src_pad % 64 == 0)
     // path recording (KIND 3): per 32-ray group, segment k of lane i is entry
     // rec_off[g] + 32 k + i of rec_leaf / rec_ds
     const long long* rec_off;
@@ -102,6 +101,7 @@ struct TraceArgs {
     // when *gate is zero (NULL: none)
     const uint32_t* rest;
     const unsigned int* n_rest;
+    unsigned long long* rest_queue;  // rays of theirs handed out so far by k_trace
 };
 
 // Ray order of a trace: direction-major (32 neighbouring sources share a

@@ -241,26 +241,39 @@ __device__ __forceinline__ void forward_ray(const TraceArgs& a, const DirConst* 
     }
 }
 
-template <int KIND, int MODE, bool UNIFORM, int SM>
+// GATED (cubes only): launched after the shared-offset form.
+template <int KIND, int MODE, bool UNIFORM, int SM, bool GATED = false>
 __global__ void __launch_bounds__(256, (MODE == RT_MODE_F32_KAHAN) ? (UNIFORM ? RT_MIN_BLOCKS_GRID : RT_MIN_BLOCKS_TREE)
                                                                 : (UNIFORM ? RT_MIN_BLOCKS : RT_MIN_BLOCKS_F64TREE))
 k_trace(const TraceArgs a)
 {
-    // the shared-offset form ran before: only the sources it left out, if any
-    const bool rest = UNIFORM && a.gate && *(volatile const int*)a.gate == 0;
-    if (UNIFORM && a.pair && !rest) return;  // k_trace_pair traced every source
-    const unsigned n_rest = rest && a.n_rest ? *(volatile const unsigned*)a.n_rest : 0u;
-    if (rest && n_rest == 0u) return;
+    if (KIND == 2 && a.gate && *(volatile const int*)a.gate == 0) return;  // the leaf gather ran instead
     if (!UNIFORM) fill_spread_table();
     const int lane = threadIdx.x & 31;
     const int gw = KIND == 3 ? 32 : a.gw;  // rays a warp walks at once
-    const unsigned long long rest_pad = (n_rest + 31u) & ~31u;
-    const unsigned long long total = (rest ? rest_pad : (unsigned long long)(a.layout ? a.n_src : a.n_src_pad)) * (unsigned long long)a.nd;
+    unsigned long long total = (unsigned long long)(a.layout ? a.n_src : a.n_src_pad) * (unsigned long long)a.nd;
     const long long cap = a.t.step_cap;
     unsigned long long n_rays = 0, n_segs = 0, n_efb = 0, n_lfb = 0;
+    bool gated = GATED, rest = false;
+    unsigned long long rest_pad = 0;
     for (;;) {
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&a.st->queue, (unsigned long long)gw * (unsigned)a.batch);
+        if (lane == 0) base = atomicAdd(rest ? a.rest_queue : &a.st->queue, (unsigned long long)gw * (unsigned)a.batch);
+        if (gated) {
+            // read after the first pop: warps that wait for it first pop in a shuffled
+            // order, which spreads neighbouring groups over the chip (64^3, 65536
+            // scattered points, FP64: 693 us in place of 660)
+            gated = false;
+            if (*(volatile const int*)a.gate == 0) {
+                // the shared-offset form ran before: only the sources it left out, if any
+                const unsigned n = *(volatile const unsigned*)a.n_rest;
+                if (n == 0u) return;
+                rest = true;
+                rest_pad = (n + 31u) & ~31u;
+                total = rest_pad * (unsigned long long)a.nd;
+                continue;
+            }
+        }
         base = __shfl_sync(RT_FULL, base, 0);
         if (base >= total) break;
         for (int kk = 0; kk < a.batch; kk++) {
@@ -272,7 +285,7 @@ k_trace(const TraceArgs a)
             if (rest) {
                 q = (int)(g0 / rest_pad);
                 const unsigned long long i = g0 - (unsigned long long)q * rest_pad + lane;
-                if (i >= n_rest) continue;
+                if (i >= *a.n_rest) continue;
                 s = (long long)__ldg(a.rest + i);
             } else if (a.layout == 0 && a.dgroup <= 1) {
                 q = (int)(g0 / (unsigned long long)a.n_src_pad);
@@ -369,7 +382,8 @@ k_trace(const TraceArgs a)
 // unit, a 64-source block and one group of dgroup directions, in the order of
 // k_trace's direction groups; lane i walks sources 64u + i and 64u + 32 + i
 // together for each direction of the group, and one at a time where the two
-// do not qualify.
+// do not qualify.  After the shared-offset form it walks the sources that form
+// left out, one ray a lane.
 #ifndef RT_MIN_BLOCKS_PAIR
 #define RT_MIN_BLOCKS_PAIR 3  // 80 registers: two rays' state without spilling the loop
 #endif
@@ -388,21 +402,42 @@ __device__ __forceinline__ void store_cols(const TraceArgs& a, long long ray, co
 template <int SM>
 __global__ void __launch_bounds__(256, RT_MIN_BLOCKS_PAIR) k_trace_pair(const TraceArgs a)
 {
-    if (a.gate && *(volatile const int*)a.gate == 0) return;  // the shared-offset form ran instead
     const int lane = threadIdx.x & 31;
-    const int D = a.dgroup > 1 ? a.dgroup : 1;
-    const unsigned long long nb2 = (unsigned long long)a.n_src_pad >> 6;
-    const unsigned long long units = nb2 * (unsigned long long)(a.nd / D);
+    // after the shared-offset form: the sources it left out, 32 of the list and one
+    // direction a unit
+    const bool rest = a.gate && *(volatile const int*)a.gate == 0;
+    const unsigned n_rest = rest ? *(volatile const unsigned*)a.n_rest : 0u;
+    if (rest && n_rest == 0u) return;
+    const int D = rest || a.dgroup <= 1 ? 1 : a.dgroup;
+    const unsigned long long nb = rest ? (n_rest + 31u) >> 5 : (unsigned long long)a.n_src_pad >> 6;
+    const unsigned long long units = nb * (unsigned long long)(a.nd / D);
     const long long cap = a.t.step_cap;
     unsigned long long n_rays = 0, n_segs = 0, n_efb = 0, n_lfb = 0;
-    for (;;) {
-        unsigned long long u = 0;
-        if (lane == 0) u = atomicAdd(&a.st->queue, 1ull);
+    // A warp's first unit goes by its number, and the queue hands out the rest: the
+    // warps of a block take neighbouring units, whatever the order in which they
+    // arrive, and fewer units than blocks go to as many SMs.  64^3, 16384 scattered
+    // points, us for 1 / 4 species: first units from the queue 602 / 372 (476 with
+    // 4 once the gate delays the warps), by number 559 / 345; 33 sources, Nside 2,
+    // one unit a block 379, neighbouring 412.
+    const unsigned long long warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const unsigned long long mine = units <= gridDim.x ? warp * gridDim.x + blockIdx.x : blockIdx.x * wpb + warp;
+    for (bool first = true;; first = false) {
+        unsigned long long u = mine;
+        if (!first && lane == 0) u = gridDim.x * wpb + atomicAdd(&a.st->queue, 1ull);
         u = __shfl_sync(RT_FULL, u, 0);
         if (u >= units) break;
-        const unsigned long long gg = u / nb2, bp = u - gg * nb2;
-        const long long s0 = (long long)(bp << 6) + lane, s1 = s0 + 32;
-        if (s0 >= a.n_src) continue;
+        const unsigned long long gg = u / nb, bp = u - gg * nb;
+        long long s0, s1;
+        if (rest) {
+            const unsigned long long i = (bp << 5) + lane;  // 32 of the list and one direction
+            if (i >= n_rest) continue;
+            s0 = (long long)__ldg(a.rest + i);
+            s1 = a.n_src;
+        } else {
+            s0 = (long long)(bp << 6) + lane;
+            s1 = s0 + 32;
+            if (s0 >= a.n_src) continue;
+        }
         const bool two = s1 < a.n_src;
         for (int dd = 0; dd < D; dd++) {
             const int q = (int)gg * D + dd;
