@@ -858,7 +858,11 @@ static size_t round256(size_t v) { return (v + 255) / 256 * 256; }
 static int padded_species(int S) { return S <= 1 ? 1 : S <= 2 ? 2 : S <= 4 ? 4 : 8; }
 
 // Tables and check results of a call, laid out from p (sizes only if p is
-// null): the bytes they take.  A sixteenth of the sources may be left out.
+// null): the bytes they take.  A sixteenth of the sources may be left out (the form
+// gains beyond that: 4 species, F32-Kahan, of a 64^3 cube a 16th 270 us against 1744
+// walked, a quarter 438 / 1870; FP64 2455 / 5067, 3442 / 5591.  The line keeps
+// the list a quarter byte a source, and is what the vote of 32 can tell from
+// scattered points).
 struct BeamScratch {
     BeamTables tab;
     BeamRef* ref;
@@ -980,15 +984,42 @@ int launch_adjoint_gather(rt_octree* t, const TraceArgs& a, int mode, cudaStream
     return RT_OK;
 }
 
+// Blocks of 32^3 leaves n_src consecutive leaves of a cube of level L may touch.
+static long long beam_blocks_of(int L, int64_t n_src)
+{
+    return std::min<long long>(1ll << (3 * (L - 5)), (n_src + 32767) / 32768 + 1);
+}
+
+// True where the form pays, us of it and of the walk, sources at leaf centres.
+//
+// F32-Kahan: sources in a sixteenth of the leaves or more: 4 species, an eighth of
+// a 32^3 cube 45 / 59, a sixteenth 45 / 57; of 64^3 78 / 102, of 256^3 1408 / 3086.  It
+// gains below that too (256^3, a 64th: 520 / 805), but scattered points
+// pay for the vote (12 us), of which a smaller call is a larger part.
+//
+// FP64 is bound by its FP64 operations in both forms, and this one computes whole
+// 32^3 blocks: at most 1.5 leaves computed a source (5 to 8 species: 1.2), and enough
+// rays to fill the chip.  64^3 at 1.25, 1.5 and 2 leaves a source: 1 species 381 /
+// 731, 246 / 404, 190 / 235; 4 species 1252 / 1445, 782 / 827, 544 / 528; 8 species
+// 2430 / 2393, 1501 / 1261, 1041 / 1041.  32^3, 1 species, every leaf (3.9e5 rays): 92 /
+// 88 on densities in L2, 95 / 122 on new ones; half of them (2.0e5) 92 / 72 and
+// 203 / 280 at Nside 2, a quarter 92 / 61 and 201 / 156.
+static bool beam_pays(int L, int64_t n_src, int nd, int S, int mode, int64_t n_leaves)
+{
+    if (n_src * 16 < n_leaves) return false;
+    if (mode != RT_MODE_FP64) return true;
+    const long long done = beam_blocks_of(L, n_src) * 32768;
+    return n_src * nd >= (1ll << 18) && (S > 4 ? done * 5 <= n_src * 6 : done * 2 <= n_src * 3);
+}
+
 // Bytes the shared-offset trace needs on this octree, 0 when its shape does
-// not admit it: a cube of at least 32^3 leaves, sources in at least a sixteenth
-// of them (the densities are copied once per call, a leaf's worth of traffic
-// against a ray's N/2 segments a source and direction), the default step cap
-// and tables of at most 256 MB.
+// not admit it: a cube of at least 32^3 leaves (its rows fill a warp), a call
+// that it is worth for, the default step cap and tables of at most 256 MB.
 size_t beam_bytes(const rt_octree* t, int64_t n_src, int nd, int S, int mode)
 {
     const int L = t->uniform_allowed ? t->dev.uniform_level : -1;
-    if (L < 5 || n_src < 32 || n_src > t->dev.n || n_src * 16 < t->dev.n || t->dev.step_cap < t->default_cap) return 0;
+    if (L < 5 || n_src < 32 || n_src > t->dev.n || !beam_pays(L, n_src, nd, S, mode, t->dev.n) || t->dev.step_cap < t->default_cap)
+        return 0;
     const size_t tab = beam_scratch(nullptr, nd, L, n_src, mode, false, nullptr);
     if (tab > (256ull << 20) + (size_t)n_src / 2) return 0;
     return tab + 2 * round256((size_t)t->dev.n * padded_species(S) * (mode == RT_MODE_FP64 ? 8 : 4));
@@ -1054,7 +1085,7 @@ int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check,
     g.field[1] = rows[1];
     g.nq = a.nd;
     g.dgroup = a.dgroup > 1 ? a.dgroup : 1;
-    g.blocks = std::min<long long>(1ll << (3 * (L - 5)), (a.n_src + 32767) / 32768 + 1);
+    g.blocks = beam_blocks_of(L, a.n_src);
     const int op = epilogue ? kBeamEpilogue : kBeamColumns;
     cudaError_t e = beam_setup(a, mode, b, b.most, 2, s);
     if (e == cudaSuccess) {

@@ -42,6 +42,8 @@ def _sources(keys, lev, how, rng):
         return c + (np.array([7 / 32, -11 / 32, 3 / 64]) + np.array([3, 5, -7]) * 2.0 ** -35) * h
     if how == "range":           # part of the leaves: ragged, not aligned to a block of any kind
         return c[n // 5 + 3:n // 2 + 18]
+    if how == "most":            # ragged at both ends, few leaves outside
+        return c[n // 50 + 3:n - n // 40 - 11]
     if how == "some_moved":      # some sources elsewhere, the first among them: the walk traces those
         idx = np.concatenate([[0, 1, 33, n - 1], rng.integers(0, n, n // 40)])
         c[idx] += (rng.random((idx.size, 3)) - 0.5) * 0.9 * h
@@ -89,6 +91,15 @@ def test_columns_equal_the_walk(rt, level, S, nside, dens, how, mode):
         r = torch.cat([rt.trace_epilogue(tree, s, nside, d, kind, [1.0] * S, 0.05, mode=mode) for s in src.split(cut)])
         torch.testing.assert_close(e, r, rtol=1e-13, atol=1e-13)
     tree.close()
+
+
+@pytest.mark.parametrize("level,S,nside,dens,how", [
+    (5, 1, 2, "f64", "centres"), (5, 2, 2, "f32", "offset"), (5, 3, 2, "f32", "some_moved"), (5, 8, 2, "f64", "last_place"),
+    (6, 2, 1, "f32", "most"), (6, 4, 1, "f64", "most"), (6, 6, 2, "f32", "most")])
+def test_fp64_columns_equal_the_walk(rt, level, S, nside, dens, how):
+    """FP64 calls large enough for the form (a quarter million rays, few leaves
+    computed in vain), ragged ranges among them."""
+    test_columns_equal_the_walk(rt, level, S, nside, dens, how, "fp64")
 
 
 @pytest.mark.parametrize("level,S,n_src,mode", [(5, 1, 2048, "f32k"), (5, 4, 32768, "fp64"), (6, 4, 16384, "f32k"), (6, 3, 16411, "f32k")])
