@@ -128,15 +128,24 @@ int rt_healpix_dirs(int nside, double* h_out);
  * The first call for a given nside on a device uploads its direction table
  * (an allocation); make that call outside CUDA graph capture.
  * On a full cube of equal-level leaves (32^3 or more), sources in consecutive
- * leaves (Morton order), at least a sixteenth of them, that share one offset
- * inside their leaf (leaf centres, for example) take no walk: every ray of a
- * direction has the same steps, and the columns are summed from step tables
- * and a row-ordered copy of the densities, bit for bit those of the walk.  The
- * sources are checked on the device; those elsewhere (all, if over a sixteenth
- * of them) are walked.  The handle keeps the tables and the copies (two of
- * n_leaves x 1, 2, 4 or 8 values), allocated by the first such call and grown
- * when a later one needs more; without memory for them, or on a stream under
- * capture, every source is walked. */
+ * leaves (Morton order) that share one offset inside their leaf (leaf centres,
+ * for example) take no walk: every ray of a direction has the same steps, and
+ * the columns are summed from step tables and a row-ordered copy of the
+ * densities, bit for bit those of the walk.  At least a sixteenth of the leaves
+ * must have a source; RT_MODE_FP64 asks for most of each 32^3-leaf block and at
+ * least 2^18 rays.  The sources are checked on the device; those elsewhere (all, if
+ * over a sixteenth of them) are walked.
+ * Memory: every call of that shape, whatever its sources turn out to be, takes
+ * two copies of the densities (n_leaves x 1, 2, 4 or 8 values each) and a
+ * quarter byte and a bit a source in the order of `stream`, and gives them back
+ * behind its last kernel, without waiting for the device.  They come from a pool
+ * of the library's own on the device, which keeps what is given back for the next
+ * call until the last octree that used it is destroyed (with
+ * rt_trace_columns_host: until its release), or until a cudaMalloc of the process
+ * needs the room.  The handle keeps the step tables (at most 256 MB; 12
+ * directions of a 512^3 cube 1.3 MB).  Without memory, or on a stream under
+ * capture, every source is walked; a capture of another stream is not
+ * disturbed. */
 int rt_trace_columns(const rt_octree* tree, const double* d_src, int64_t n_src, int nside,
                      const void* d_dens, int n_species, int dens_dtype, int mode,
                      void* d_out, void* stream);
@@ -156,9 +165,10 @@ int rt_trace_columns(const rt_octree* tree, const double* d_src, int64_t n_src, 
  *     or cudaHostRegister) let the copies run as DMA.
  *   h_stats: optional; receives the trace's statistics.
  *   stream: the stream the traces run on (two more are created inside).
- * Device buffers (the octree, densities, all sources and two column
- * chunks), the two copy streams and the events are kept per device between
- * calls and grow on demand; rt_trace_columns_host_release frees them.  Calls
+ * Device buffers (the octree, densities, all sources, two column chunks and
+ * the step tables of rt_trace_columns's form for shared offsets), the two copy
+ * streams and the events are kept per device between calls and grow on demand;
+ * rt_trace_columns_host_release frees them.  Calls
  * are serialized by a process-wide lock.  Returns RT_ERR_OOM if the buffers
  * do not fit, the code of the first faulting ray if a ray faulted (its
  * columns are zero), and the rt_build_octree codes for a malformed octree. */

@@ -235,6 +235,7 @@ void rt_destroy_octree(rt_octree* t)
     if (t->st) cudaFree(t->st);
     if (t->adj_tab) cudaFree(t->adj_tab);
     if (t->fwd_tab && !t->fwd_tab_lent) cudaFree(t->fwd_tab);
+    if (t->fwd_pool) beam_pool_leave(t->device);
     free(t);
 }
 
@@ -313,10 +314,10 @@ int rt::trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_sr
     if (a.t.uniform_level >= 0) a.dgroup = output_dgroup(a.nd, n_species, mode);
     // sources at one offset in consecutive leaves of a cube: no walk at all;
     // the walk below then traces those the device finds elsewhere
-    bool beam = false;
-    st = launch_beam((rt_octree*)t, a, mode, false, check, s, &beam);
+    BeamCall beam;
+    st = launch_beam((rt_octree*)t, a, mode, false, check, s, beam);
     if (st != RT_OK) return st;
-    if (!beam && check) {
+    if (!beam.p && check) {
         st = check_densities(d_dens, t->dev.n, n_species, a.dens_f64, 0, t->st, s);
         if (st != RT_OK) return st;
     }
@@ -327,7 +328,7 @@ int rt::trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_sr
     if (a.pair) a.n_src_pad = (n_src + 63) / 64 * 64;
     const int fit = a.pair ? occupancy_pair(n_species, g_block)
                            : occupancy_fwd(0, mode, n_species, a.t.uniform_level >= 0, g_block);
-    if (!beam && cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
+    if (!beam.p && cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
         return cuda_error("rt_trace_columns: queue reset");
     const int grid = grid_for(fit);
     spread_rays(a, (long long)grid * (g_block / 32));

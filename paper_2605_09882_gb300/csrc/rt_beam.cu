@@ -31,6 +31,8 @@
 // run-axis cells passed before it, and its segment lengths.  For every axis b
 // and every r, P_b[r] is the first step that is more than r cells from the
 // start on b, and C_b[r] the same in runs for the two other axes.
+#include <mutex>
+
 #include "rt_host.h"
 #include "rt_kernels.cuh"
 
@@ -857,51 +859,55 @@ static size_t round256(size_t v) { return (v + 255) / 256 * 256; }
 
 static int padded_species(int S) { return S <= 1 ? 1 : S <= 2 ? 2 : S <= 4 ? 4 : 8; }
 
-// Tables and check results of a call, laid out from p (sizes only if p is
-// null): the bytes they take.  A sixteenth of the sources may be left out (the form
-// gains beyond that: 4 species, F32-Kahan, of a 64^3 cube a 16th 270 us against 1744
-// walked, a quarter 438 / 1870; FP64 2455 / 5067, 3442 / 5591.  The line keeps
-// the list a quarter byte a source, and is what the vote of 32 can tell from
-// scattered points).
+// Scratch of a call in two parts, laid out from p (the tables, which a later
+// call finds there, so at places that do not depend on n_src) and from v (the
+// check's results); sizes only if p is null.  A sixteenth of the sources may be left
+// out (the form gains beyond that: 4 species, F32-Kahan, of a 64^3 cube a 16th 270 us against
+// 1744 walked, a quarter 438 / 1870; FP64 2455 / 5067, 3442 / 5591.  The line
+// keeps the list a quarter byte a source, and is what the vote of 32 can tell
+// from scattered points).
 struct BeamScratch {
     BeamTables tab;
     BeamRef* ref;
     uint32_t *out, *rest;
     unsigned long long* queue;
     unsigned int most;
+    size_t kept, call;  // bytes of the two parts
 };
 
-static size_t beam_scratch(char* p, int nd, int L, int64_t n_src, int mode, bool adjoint, BeamScratch* b)
+static BeamScratch beam_scratch(char* p, char* v, int nd, int L, int64_t n_src, int mode, bool adjoint)
 {
+    BeamScratch b;
+    memset(&b, 0, sizeof b);
     const int N = 1 << L;
     const int lcap = (3 * N + 3 + 15) / 16 * 16, pcap = (N + 1 + 3) / 4 * 4;
     const size_t rsz = mode == RT_MODE_FP64 ? sizeof(BeamRun<double>) : sizeof(BeamRun<float>);
-    const unsigned int most = (unsigned int)(n_src / 16);
     const size_t steps = adjoint ? (size_t)nd * lcap : 0;
-    // the tables first, at places that do not depend on n_src: a later call finds them there
     const size_t bytes[] = {sizeof(BeamRef), (size_t)nd * sizeof(int4), (size_t)nd * lcap * rsz, (size_t)nd * lcap * 4,
                             (size_t)nd * 3 * pcap * 4, (size_t)nd * 3 * pcap * 4, steps * 4,
-                            steps * (mode == RT_MODE_FP64 ? 8 : 4), (size_t)(adjoint ? nd : 2) * 8,
-                            (size_t)((n_src + 31) / 32) * 4, (size_t)most * 4};
-    size_t at[12] = {0};
-    for (int i = 0; i < 11; i++) at[i + 1] = at[i] + round256(bytes[i]);
+                            steps * (mode == RT_MODE_FP64 ? 8 : 4), (size_t)(adjoint ? nd : 2) * 8};
+    size_t at[10] = {0};
+    for (int i = 0; i < 9; i++) at[i + 1] = at[i] + round256(bytes[i]);
+    b.most = (unsigned int)(n_src / 16);
+    const size_t list = round256((size_t)((n_src + 31) / 32) * 4);
+    b.kept = at[9];
+    b.call = list + round256((size_t)b.most * 4);
+    b.tab.lcap = lcap;
+    b.tab.pcap = pcap;
     if (p) {
-        b->ref = (BeamRef*)(p + at[0]);
-        b->tab.info = (int4*)(p + at[1]);
-        b->tab.run = p + at[2];
-        b->tab.fb = (int*)(p + at[3]);
-        b->tab.P = (int*)(p + at[4]);
-        b->tab.C = (int*)(p + at[5]);
-        b->tab.D = adjoint ? (int*)(p + at[6]) : nullptr;
-        b->tab.ds = adjoint ? p + at[7] : nullptr;
-        b->queue = (unsigned long long*)(p + at[8]);
-        b->out = (uint32_t*)(p + at[9]);
-        b->rest = (uint32_t*)(p + at[10]);
-        b->tab.lcap = lcap;
-        b->tab.pcap = pcap;
-        b->most = most;
+        b.ref = (BeamRef*)(p + at[0]);
+        b.tab.info = (int4*)(p + at[1]);
+        b.tab.run = p + at[2];
+        b.tab.fb = (int*)(p + at[3]);
+        b.tab.P = (int*)(p + at[4]);
+        b.tab.C = (int*)(p + at[5]);
+        b.tab.D = adjoint ? (int*)(p + at[6]) : nullptr;
+        b.tab.ds = adjoint ? p + at[7] : nullptr;
+        b.queue = (unsigned long long*)(p + at[8]);
+        b.out = (uint32_t*)v;
+        b.rest = (uint32_t*)(v + list);
     }
-    return at[11];
+    return b;
 }
 
 // Sources of 32 at the commonest offset below which a form that may leave out a
@@ -943,8 +949,8 @@ bool gather_applies(const rt_octree* t, const TraceArgs& a)
 int launch_adjoint_gather(rt_octree* t, const TraceArgs& a, int mode, cudaStream_t s)
 {
     const size_t tsz = mode == RT_MODE_FP64 ? 8 : 4;
-    const size_t t_bytes = beam_scratch(nullptr, a.nd, a.t.uniform_level, a.n_src, mode, true, nullptr);
-    const size_t need = t_bytes + (size_t)a.n_src * a.S * tsz;
+    const BeamScratch sz = beam_scratch(nullptr, nullptr, a.nd, a.t.uniform_level, a.n_src, mode, true);
+    const size_t need = sz.kept + sz.call + (size_t)a.n_src * a.S * tsz;
     if (t->adj_tab_bytes < need) {
         if (t->adj_tab) {
             cudaStreamSynchronize(s);
@@ -962,11 +968,10 @@ int launch_adjoint_gather(rt_octree* t, const TraceArgs& a, int mode, cudaStream
     BeamArgs g;
     memset(&g, 0, sizeof g);
     g.t = a;
-    BeamScratch b;
-    beam_scratch((char*)t->adj_tab, a.nd, a.t.uniform_level, a.n_src, mode, true, &b);
+    const BeamScratch b = beam_scratch((char*)t->adj_tab, (char*)t->adj_tab + sz.kept, a.nd, a.t.uniform_level, a.n_src, mode, true);
     g.tab = b.tab;
     g.queue = b.queue;
-    char* gl = (char*)t->adj_tab + t_bytes;
+    char* gl = (char*)t->adj_tab + sz.kept + sz.call;
     g.field[0] = g.field[1] = gl;
     g.nq = g.dgroup = 1;
     const int L = a.t.uniform_level;
@@ -1012,17 +1017,97 @@ static bool beam_pays(int L, int64_t n_src, int nd, int S, int mode, int64_t n_l
     return n_src * nd >= (1ll << 18) && (S > 4 ? done * 5 <= n_src * 6 : done * 2 <= n_src * 3);
 }
 
-// Bytes the shared-offset trace needs on this octree, 0 when its shape does
-// not admit it: a cube of at least 32^3 leaves (its rows fill a warp), a call
-// that it is worth for, the default step cap and tables of at most 256 MB.
+// Bytes of tables the shared-offset trace keeps on this octree, 0 when its
+// shape does not admit it: a cube of at least 32^3 leaves (its rows fill a
+// warp), a call that it is worth for, the default step cap and tables of at most
+// 256 MB.
 size_t beam_bytes(const rt_octree* t, int64_t n_src, int nd, int S, int mode)
 {
     const int L = t->uniform_allowed ? t->dev.uniform_level : -1;
     if (L < 5 || n_src < 32 || n_src > t->dev.n || !beam_pays(L, n_src, nd, S, mode, t->dev.n) || t->dev.step_cap < t->default_cap)
         return 0;
-    const size_t tab = beam_scratch(nullptr, nd, L, n_src, mode, false, nullptr);
-    if (tab > (256ull << 20) + (size_t)n_src / 2) return 0;
-    return tab + 2 * round256((size_t)t->dev.n * padded_species(S) * (mode == RT_MODE_FP64 ? 8 : 4));
+    const size_t kept = beam_scratch(nullptr, nullptr, nd, L, n_src, mode, false).kept;
+    return kept > (256ull << 20) ? 0 : kept;
+}
+
+// Memory of the shared-offset trace comes from a pool of the device, in the order
+// of the stream: a call takes what it needs (two row copies of the
+// densities, the check's results) and gives it back behind its last kernel, so
+// no call waits for the device, and between calls a handle holds its tables
+// alone.  The pool keeps what is given back for the next call (a 4.3 GB block: 1.5
+// us, against 2.5 ms from the device and 4.3 to return it) while a handle or
+// the host call's buffers use it, and returns all of it with the last of them;
+// an allocation by cudaMalloc that does not fit takes it from the pool before that.
+// It is never used by way of another stream's unfinished work (no stream
+// waits for another on account of memory).
+namespace {
+struct Pool {
+    cudaMemPool_t pool = nullptr;
+    int users = 0;
+};
+std::mutex g_pool_mu;
+Pool g_pool[64];
+}  // namespace
+
+// An allocation here is safe beside another stream's capture, but the runtime
+// refuses it, and breaks that capture, unless this thread asks for relaxed checks.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+bool beam_pool_join(int dev)
+{
+    if (dev < 0 || dev >= 64) return false;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    Pool& p = g_pool[dev];
+    if (!p.pool) {
+        RelaxedCapture relaxed;
+        cudaMemPoolProps props;
+        memset(&props, 0, sizeof props);
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        unsigned long long keep = ~0ull;
+        int no = 0;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess) {
+            cudaGetLastError();
+            if (pool) cudaMemPoolDestroy(pool);
+            return false;
+        }
+        p.pool = pool;
+    }
+    p.users++;
+    return true;
+}
+
+void beam_pool_leave(int dev)
+{
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (--g_pool[dev].users == 0) cudaMemPoolTrimTo(g_pool[dev].pool, 0);
+}
+
+// `bytes` of the device's pool on `s`, null if there is no room.
+static void* beam_alloc(int dev, size_t bytes, cudaStream_t s)
+{
+    RelaxedCapture relaxed;
+    void* p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, bytes, g_pool[dev].pool, s) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
+BeamCall::~BeamCall()
+{
+    if (!p) return;
+    RelaxedCapture relaxed;
+    cudaFreeAsync(p, s);
 }
 
 template <int MODE, int SM>
@@ -1038,49 +1123,44 @@ static cudaError_t go_trace(const BeamArgs& g, void* const rows[2], bool check, 
 }
 
 // Enqueues the shared-offset forward trace (with the density check) or
-// epilogue on `s`, if the call's shape admits it; ran tells whether it did.
+// epilogue on `s`, if the call's shape admits it; call.p tells whether it did.
 // It sets a's gate and list of left-out sources for the walk launched after
-// it, and resets that walk's queue.  Its scratch belongs to the handle: a captured stream, or no memory for it, leaves the
-// call to the walk.
-int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check, cudaStream_t s, bool* ran)
+// it (call holds what that walk reads, until it is destroyed), and resets that
+// walk's queue.  A captured stream, or no memory, leaves the call to the walk.
+int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check, cudaStream_t s, BeamCall& call)
 {
-    *ran = false;
-    const size_t need = beam_bytes(t, a.n_src, a.nd, a.S, mode);
-    if (!need || a.t.uniform_level < 0) return RT_OK;
+    const size_t kept = beam_bytes(t, a.n_src, a.nd, a.S, mode);
+    if (!kept || a.t.uniform_level < 0) return RT_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
         return RT_OK;
     }
-    if (t->fwd_tab_bytes < need) {
+    if (!t->fwd_pool && !(t->fwd_pool = beam_pool_join(t->device))) return RT_OK;
+    const int L = a.t.uniform_level, SM = padded_species(a.S);
+    const size_t row_bytes = round256((size_t)t->dev.n * SM * (mode == RT_MODE_FP64 ? 8 : 4));
+    const BeamScratch sz = beam_scratch(nullptr, nullptr, a.nd, L, a.n_src, mode, false);
+    if (t->fwd_tab_bytes < kept) {
         if (t->fwd_tab_lent) return RT_OK;
-        if (t->fwd_tab) {
-            cudaStreamSynchronize(s);
-            cudaFree(t->fwd_tab);
-            t->fwd_tab = nullptr;
-            t->fwd_tab_bytes = 0;
-        }
-        if (cudaMalloc(&t->fwd_tab, need) != cudaSuccess) {
-            cudaGetLastError();
-            t->fwd_tab = nullptr;
-            return RT_OK;
-        }
-        t->fwd_tab_bytes = need;
+        BeamCall old{t->fwd_tab, s};
+        t->fwd_tab_bytes = 0;
+        if (!(t->fwd_tab = beam_alloc(t->device, kept, s))) return RT_OK;
+        t->fwd_tab_bytes = kept;
         cudaMemsetAsync(t->fwd_tab, 0, sizeof(BeamRef), s);  // no tables yet
     }
-    const int L = a.t.uniform_level, SM = padded_species(a.S);
-    const size_t t_bytes = beam_scratch(nullptr, a.nd, L, a.n_src, mode, false, nullptr);
-    const size_t row_bytes = round256((size_t)t->dev.n * SM * (mode == RT_MODE_FP64 ? 8 : 4));
+    char* v = (char*)beam_alloc(t->device, sz.call + 2 * row_bytes, s);
+    if (!v) return RT_OK;
+    call.p = v;
+    call.s = s;
     BeamArgs g;
     memset(&g, 0, sizeof g);
     g.t = a;
-    BeamScratch b;
-    beam_scratch((char*)t->fwd_tab, a.nd, L, a.n_src, mode, false, &b);
+    const BeamScratch b = beam_scratch((char*)t->fwd_tab, v, a.nd, L, a.n_src, mode, false);
     g.tab = b.tab;
     g.queue = b.queue;
     g.ref = b.ref;
     g.out = b.out;
-    void* rows[2] = {(char*)t->fwd_tab + t_bytes, (char*)t->fwd_tab + t_bytes + row_bytes};
+    void* rows[2] = {v + sz.call, v + sz.call + row_bytes};
     g.field[0] = rows[0];
     g.field[1] = rows[1];
     g.nq = a.nd;
@@ -1101,7 +1181,6 @@ int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check,
     a.rest = b.rest;
     a.n_rest = &b.ref->n_rest;
     a.rest_queue = b.queue + 1;
-    *ran = true;
     return RT_OK;
 }
 

@@ -88,10 +88,10 @@ extern "C" int rt_trace_epilogue(const rt_octree* t, const double* d_src, int64_
     if (h_epi->kind != RT_EPI_ATTENUATION &&
         cudaMemsetAsync(d_out, 0, sizeof(double) * (size_t)n_src, s) != cudaSuccess)
         return cuda_error("rt_trace_epilogue: clear");
-    bool beam = false;
-    st = launch_beam((rt_octree*)t, a, mode, true, true, s, &beam);
+    BeamCall beam;
+    st = launch_beam((rt_octree*)t, a, mode, true, true, s, beam);
     if (st != RT_OK) return st;
-    if (!beam && (st = check_densities(d_dens, t->dev.n, n_species, a.dens_f64, 0, t->st, s)) != RT_OK) return st;
+    if (!beam.p && (st = check_densities(d_dens, t->dev.n, n_species, a.dens_f64, 0, t->st, s)) != RT_OK) return st;
     int block, bps, groups;
     launch_shape(&block, &bps, &groups);
     int dev = 0;
@@ -99,7 +99,7 @@ extern "C" int rt_trace_epilogue(const rt_octree* t, const double* d_src, int64_
     const int fit = occupancy_epi(mode, n_species, a.t.uniform_level >= 0, block);
     const int grid = sm_count_of(dev) * std::max(1, bps > 0 ? std::min(bps, fit) : fit);
     spread_rays(a, (long long)grid * (block / 32));
-    if ((!beam && cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess) ||
+    if ((!beam.p && cudaMemsetAsync(&t->st->queue, 0, sizeof(unsigned long long), s) != cudaSuccess) ||
         launch_epilogue(a, mode, block, grid, s) != cudaSuccess)
         return cuda_error("rt_trace_epilogue: launch");
     if (h_epi->kind != RT_EPI_ATTENUATION) {

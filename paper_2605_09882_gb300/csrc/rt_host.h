@@ -32,10 +32,21 @@ int trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_src, i
 // argument checks and TraceArgs of the single-octree trace entry points
 int prepare_trace(const rt_octree* t, const double* d_src, int64_t n_src, int nside, int S, int mode,
                   TraceArgs& a, const char* who);
-// shared-offset trace of a cube (rt_beam.cu): the scratch it needs (0: the
-// shape does not admit it) and its launch, with the density check if asked
+// shared-offset trace of a cube (rt_beam.cu): the tables it keeps (bytes; 0: the
+// shape does not admit it), the memory of one call (p null: the form did not
+// run; given back to the pool, in the order of s, when destroyed) and its launch,
+// with the density check if asked
 size_t beam_bytes(const rt_octree* t, int64_t n_src, int nd, int S, int mode);
-int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check, cudaStream_t s, bool* ran);
+struct BeamCall {
+    void* p = nullptr;
+    cudaStream_t s = nullptr;
+    ~BeamCall();
+};
+int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check, cudaStream_t s, BeamCall& call);
+// a user of the pool that memory comes from (a handle, the host call's buffers)
+// comes and goes
+bool beam_pool_join(int dev);
+void beam_pool_leave(int dev);
 // leaf-gather adjoint (rt_beam.cu): whether the call's shape admits it, and
 // its launch (source check, step tables, gather) on stream s
 bool gather_applies(const rt_octree* t, const TraceArgs& a);

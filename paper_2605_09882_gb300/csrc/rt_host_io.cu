@@ -14,16 +14,17 @@ using namespace rt;
 
 namespace {
 
-enum { kKeys, kLevels, kDens, kSrc, kOut0, kOut1, kRows, kBufs };
+enum { kKeys, kLevels, kDens, kSrc, kOut0, kOut1, kTab, kBufs };
 
 struct Workspace {
     void* buf[kBufs] = {};
     size_t cap[kBufs] = {};
+    bool pool = false;  // a user of the shared-offset trace's pool
     cudaStream_t up = nullptr, down = nullptr;
     cudaEvent_t dens_in = nullptr;
     std::vector<cudaEvent_t> ev;  // per chunk: source in, traced, output out
 
-    void release()
+    void release(int dev)
     {
         if (up) cudaStreamSynchronize(up);
         if (down) cudaStreamSynchronize(down);
@@ -39,6 +40,8 @@ struct Workspace {
             buf[i] = nullptr;
             cap[i] = 0;
         }
+        if (pool) beam_pool_leave(dev);
+        pool = false;
     }
 };
 
@@ -137,14 +140,15 @@ extern "C" int rt_trace_columns_host(const uint64_t* h_keys, const uint8_t* h_le
         return cuda_error(who);
     int st = rt_build_octree(keys, levels, n_leaves, h_extent, stream, &guard.tree);
     if (st != RT_OK) return st;
-    // scratch of the shared-offset trace, kept between calls (without it the
-    // handle of this call would allocate its own, or walk)
+    // step tables of the shared-offset trace, kept between calls (without them
+    // the handle of this call would make its own), and its pool's memory with them
     if (const size_t need = n_src ? beam_bytes(guard.tree, std::min(chunk, n_src), (int)nd, S, mode) : 0) {
-        const size_t had = w.cap[kRows];
-        if (reserve(w, kRows, need)) {
-            if (w.cap[kRows] != had) cudaMemsetAsync(w.buf[kRows], 0, 256, cs);  // no step tables in it yet
-            guard.tree->fwd_tab = w.buf[kRows];
-            guard.tree->fwd_tab_bytes = w.cap[kRows];
+        const size_t had = w.cap[kTab];
+        if (!w.pool) w.pool = beam_pool_join(dev);
+        if (w.pool && reserve(w, kTab, need)) {
+            if (w.cap[kTab] != had) cudaMemsetAsync(w.buf[kTab], 0, 256, cs);  // no step tables in it yet
+            guard.tree->fwd_tab = w.buf[kTab];
+            guard.tree->fwd_tab_bytes = w.cap[kTab];
         }
         guard.tree->fwd_tab_lent = 1;
     }
@@ -199,7 +203,7 @@ extern "C" void rt_trace_columns_host_release(void)
         int cur = 0;
         cudaGetDevice(&cur);
         cudaSetDevice(kv.first);
-        kv.second.release();
+        kv.second.release(kv.first);
         cudaSetDevice(cur);
     }
     g_ws.clear();

@@ -131,8 +131,9 @@ struct rt_octree {
     int64_t default_cap;
     void* adj_tab;           // device, owned: step tables of the leaf-gather adjoint (grown on demand)
     size_t adj_tab_bytes;
-    void* fwd_tab;           // device: step tables and row-layout densities of the shared-offset trace
+    void* fwd_tab;           // device: step tables of the shared-offset trace
     size_t fwd_tab_bytes;
+    int fwd_pool;            // a user of its pool
     int fwd_tab_lent;        // fwd_tab belongs to the caller that built the handle
     unsigned long long gen;  // build number, unique in the process (a reused address is another tree)
 };

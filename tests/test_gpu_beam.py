@@ -158,6 +158,56 @@ def test_captured_call_walks(rt):
     tree.close()
 
 
+@pytest.mark.parametrize("how", ["centres", "scattered"])
+def test_memory_between_calls(rt, how):
+    """A handle that has traced keeps its tables, not the row copies of the
+    densities (two of 134 MB here): an allocation of all that is free and
+    half of them besides fits, and the next call still gives the same columns."""
+    import torch
+    keys, lev = uniform_octree(7)
+    tree = rt.Octree(_dev(keys), _dev(lev))
+    src = _dev(_sources(keys, lev, "centres", None) if how == "centres" else np.random.default_rng(5).random((keys.shape[0], 3)))
+    d = torch.rand((keys.shape[0], 8), device="cuda", dtype=torch.float64)
+    out = rt.trace_columns(tree, src, 1, d, "fp64")
+    want = out.clone()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    held = torch.empty(torch.cuda.mem_get_info()[0] + (128 << 20), dtype=torch.uint8, device="cuda")
+    del held
+    torch.cuda.empty_cache()
+    assert torch.equal(rt.trace_columns(tree, src, 1, d, "fp64", out=out), want)
+    tree.close()
+
+
+def test_first_call_beside_a_capture(rt):
+    """A handle's first call, and one that needs larger tables, on a stream of its
+    own while another stream is captured in the default mode: the capture stands
+    and both results are right."""
+    import torch
+    keys, lev = uniform_octree(5)
+    src = _dev(_sources(keys, lev, "centres", None))
+    d = torch.rand((keys.shape[0], 4), device="cuda")
+    other = rt.Octree(_dev(keys), _dev(lev))  # loads the kernels and the directions
+    want = [rt.trace_columns(other, src, ns, d) for ns in (1, 2)]
+    tree = rt.Octree(_dev(keys), _dev(lev))
+    out = [torch.zeros_like(w) for w in want]
+    x = torch.zeros(1000, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        x += 1
+        for ns in (1, 2):
+            rt.trace_columns(tree, src, ns, d, out=out[ns - 1], stream=side)
+        x += 1
+    g.replay()
+    torch.cuda.synchronize()
+    assert bool((x == 2).all())
+    assert all(torch.equal(a, b) for a, b in zip(out, want))
+    tree.close()
+    other.close()
+
+
 @pytest.mark.parametrize("n_src,nside", [(1, 1), (1, 8), (7, 4), (31, 2), (33, 1), (100, 2)])
 @pytest.mark.parametrize("mode", ["f32k", "fp64"])
 def test_few_rays_equal_many(rt, n_src, nside, mode):
