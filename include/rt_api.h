@@ -143,7 +143,7 @@ int rt_healpix_dirs(int nside, double* h_out);
  * call until the last octree that used it is destroyed (with
  * rt_trace_columns_host: until its release), or until a cudaMalloc of the process
  * needs the room.  The handle keeps the step tables (at most 256 MB; 12
- * directions of a 512^3 cube 1.3 MB).  Without memory, or on a stream under
+ * directions of a 512^3 cube 0.8 MB).  Without memory, or on a stream under
  * capture, every source is walked; a capture of another stream is not
  * disturbed. */
 int rt_trace_columns(const rt_octree* tree, const double* d_src, int64_t n_src, int nside,

@@ -910,12 +910,6 @@ static BeamScratch beam_scratch(char* p, char* v, int nd, int L, int64_t n_src, 
     return b;
 }
 
-// Sources of 32 at the commonest offset below which a form that may leave out a
-// sixteenth is not tried.  With a sixteenth elsewhere at random, fewer than 24
-// agree once in 9,000 calls (and the walk then does what the form would have);
-// with half elsewhere, more than 23 once in 280.
-constexpr int kBeamVotes = 24;
-
 // Enqueues the source check (most: sources that may be left out) and the tables,
 // and resets the queues.
 static cudaError_t beam_setup(const TraceArgs& a, int mode, const BeamScratch& b, unsigned int most, int queues, cudaStream_t s)

@@ -8,7 +8,7 @@ import pytest
 
 import oracle
 import synth
-from tinytrees import random_octree
+from tinytrees import random_octree, uniform_octree
 
 pytestmark = pytest.mark.gpu
 
@@ -145,3 +145,51 @@ def test_host_call_extent_and_fp64_densities(rt, mode):
     else:
         d = np.abs(got.numpy().astype(np.float64) - ref)
         assert (d <= RTOL * np.abs(ref) + ATOL).all()
+
+
+def test_host_call_on_cubes(rt):
+    """Cubes whose sources share an offset: no walk, but step tables that stay in
+    the call's buffers between calls.  Each call's columns and segments are those
+    of the walk (the device call with a step cap no ray reaches, which turns the form
+    off), bit for bit, whatever the call before left behind: chunks with a ragged
+    last one and one too small for the form, other densities and species, another
+    Nside, mode, level or offset and back, larger tables and smaller ones again,
+    sources of which none or only some share an offset, a density that is no number."""
+    import torch
+    rng = np.random.default_rng(41)
+    cubes = {}
+    for level in (5, 6):
+        keys, lev = uniform_octree(level)
+        h = 2.0 ** -level
+        centres = synth.leaf_centres(synth.Cloud(keys, lev, np.zeros((keys.shape[0], 1)), (1 << 21,) * 3))
+        half = np.concatenate([centres[:keys.shape[0] // 2], np.sort(rng.random((keys.shape[0] // 2, 3)), axis=0)])
+        moved = centres.copy()
+        moved[::37] += 0.3 * h
+        cubes[level] = keys, lev, dict(centres=centres, offset=centres + np.array([7, -11, 3]) * h / 32, half=half, moved=moved,
+                                       scattered=rng.random(centres.shape))
+    n6 = 1 << 18
+    calls = [(6, 2, 1, "f32k", "centres", n6 // 5), (6, 2, 1, "f32k", "centres", n6 // 5), (6, 3, 1, "f32k", "centres", 0),
+             (6, 8, 1, "f32k", "offset", n6 // 3), (6, 2, 1, "f32k", "centres", n6 - 64), (6, 1, 2, "fp64", "centres", 0),
+             (5, 4, 2, "f32k", "centres", 0), (5, 4, 1, "f32k", "offset", 4096), (5, 4, 2, "fp64", "offset", 32768),
+             (5, 4, 1, "f32k", "centres", 4096), (6, 2, 1, "f32k", "half", 0), (6, 2, 1, "f32k", "moved", n6 // 4),
+             (5, 2, 1, "f32k", "scattered", 0), (6, 2, 4, "f32k", "centres", 0), (5, 1, 1, "f32k", "centres", 1 << 14)]
+    rt.trace_columns_host_release()
+    for level, S, nside, mode, how, chunk in calls:
+        keys, lev, sources = cubes[level]
+        src = sources[how]
+        dens = rng.lognormal(0.0, 2.0, size=(keys.shape[0], S)).astype(np.float32)
+        k, l, s, d = (torch.from_numpy(a) for a in (keys.view(np.int64), lev, src, dens))
+        got, st = rt.trace_columns_host(k, l, s, nside, d, mode, chunk=chunk)
+        tree = rt.Octree(k.cuda(), l.cuda())
+        tree.set_step_cap(3 * (1 << level) + 2)
+        tree.reset_stats()
+        want = rt.trace_columns(tree, s.cuda(), nside, d.cuda(), mode).cpu()
+        walked = tree.stats()
+        tree.close()
+        assert torch.equal(got, want), (level, S, nside, mode, how, chunk)
+        assert st["status"] == 0 and (st["rays"], st["segments"]) == (walked["rays"], walked["segments"])
+    dens[1234, 0] = np.inf
+    with pytest.raises(rt.RTError) as e:
+        rt.trace_columns_host(k, l, s, 1, torch.from_numpy(dens), "f32k")
+    assert e.value.code == 7  # RT_ERR_NONFINITE
+    rt.trace_columns_host_release()
