@@ -1185,7 +1185,7 @@ __device__ __forceinline__ int walk_tree(const DevTree& t, const DirConst* __res
             const float ds = __fadd_rn(__fsub_rn(the, tih), __fsub_rn(tle, til));
             tih = the;
             til = tle;
-    vis.acc(ds);
+            vis.acc(ds);
         }
         wc.nseg++;
         // the exit axes enter the next cell, the others take the exit point; a
@@ -1225,7 +1225,7 @@ __device__ __forceinline__ int walk_tree(const DevTree& t, const DirConst* __res
                     apart |= (uint32_t)(a ^ z);
                 }
             }
-            if (!hit || (apart & ~(size - 1u)) != 0u) {
+            if ((apart & ~(size - 1u)) != 0u) {
                 const unsigned E = (e[0] ? 1u : 0u) | (e[1] ? 2u : 0u) | (e[2] ? 4u : 0u);
 #pragma unroll
                 for (int b = 0; b < 3; b++) x[b] = (c[b] ^ mir(b)) & kOnes;
