@@ -232,3 +232,25 @@ def test_few_rays_equal_many(rt, n_src, nside, mode):
     lhs, rhs = (g.double() * want.double()).sum(), (grad * dens.double()).sum()
     torch.testing.assert_close(lhs, rhs, rtol=1e-12 if mode == "fp64" else 1e-5, atol=0)
     tree.close()
+
+
+@pytest.mark.parametrize("n_src,nside", [(1, 2), (3, 8), (31, 2), (33, 1), (100, 2)])
+@pytest.mark.parametrize("mode", ["f32k", "fp64"])
+@pytest.mark.parametrize("grid", ["octree", "cube"])
+def test_few_rays_epilogue(rt, n_src, nside, mode, grid):
+    """The epilogues of a call of few rays: each ray's term is that of the same
+    ray among many, and a source's sum of them within a rounding a direction."""
+    import torch
+    from tinytrees import random_octree
+    rng = np.random.default_rng(78)
+    keys, lev = uniform_octree(4) if grid == "cube" else random_octree(rng, 1, 6, 0.35)[:2]
+    tree = rt.Octree(_dev(keys), _dev(lev))
+    dens = _dev(rng.random((keys.shape[0], 3)).astype(np.float32))
+    many = _dev(rng.random((6000, 3)))
+    for kind in ("attenuation", "av_eff", "beta"):
+        few, all_ = (rt.trace_epilogue(tree, s, nside, dens, kind, [1.0, 2.0, 0.5], 0.7, mode=mode) for s in (many[:n_src], many))
+        if kind == "attenuation":
+            assert torch.equal(few, all_[:n_src])
+        else:  # A_V,eff takes the logarithm of a mean of at least exp(-3.02 * 0.7 * 3.5 sqrt(3))
+            torch.testing.assert_close(few, all_[:n_src], rtol=12 * nside * nside * 2.0 ** -52, atol=12 * nside * nside * 2.0 ** -52)
+    tree.close()

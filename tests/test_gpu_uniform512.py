@@ -111,3 +111,15 @@ def test_adjoint_full_size_sparse_seed(setup):
     assert np.array_equal(got == 0.0, ref == 0.0)
     touched = ref > 0
     print("leaves touched", int(touched[:, 0].sum()), "max rel", float((np.abs(got - ref)[touched] / ref[touched]).max()))
+
+
+def test_walk_sampled(setup):
+    """The cube walk at level 9, which the full trace no longer takes: the
+    sampled sources alone are too few for the form that replaces it."""
+    rt, torch = setup["rt"], setup["torch"]
+    src = setup["src"][torch.from_numpy(setup["idx"]).cuda()]
+    assert src.shape[0] * 16 < setup["n"]
+    got = rt.trace_columns(setup["tree"], src, 1, setup["dens"], "f32k").double().cpu().numpy()
+    assert np.all(np.abs(got - setup["want"]) <= 1e-5 * np.abs(setup["want"]) + 1e-30)
+    got = rt.trace_columns(setup["tree"], src, 1, setup["dens"], "fp64").cpu().numpy()
+    np.testing.assert_array_equal(got, setup["want"])
