@@ -356,7 +356,8 @@ int rt_set_step_cap(rt_octree* tree, int64_t cap);
 /* Launch shape of the persistent trace kernels: threads per block (a
  * multiple of 32 in 32..256; 0 = default 256), resident blocks per SM (0 =
  * as many as fit) and 32-ray groups a warp takes per work-queue pop (1..64;
- * 0 = default 4).  Applies to later calls in this process.  The F32-Kahan
+ * 0 = default 4; a call too small to give every warp that many takes fewer,
+ * and of fewer rays).  Applies to later calls in this process.  The F32-Kahan
  * forward of rt_trace_columns on a full cube of equal-level leaves with FP32
  * densities of 1, 2, 4 or 8 species walks two rays per lane: its warps pop
  * one 64-source block and one direction group at a time, whatever

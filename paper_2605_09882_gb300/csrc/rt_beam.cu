@@ -545,12 +545,17 @@ __device__ __forceinline__ void load_run(const BeamRun<T>* __restrict__ e, int4&
 // Leaves a thread takes along the run axis (R), and blocks of kBeamWarps warps
 // an SM holds.  A longer row shares each loaded cell among more leaves and
 // spreads a run's fixed cost (its table entry, its branch, the wait for its
-// cells) over more sums; it takes registers from the warps in flight.  Columns
-// of a 256^3 cube, 4 species, F32-Kahan, in ms: R = 2 at 64 registers 25.2; 4 at
-// 128 23.2, at 96 21.5, at 80 21.0; 8 at 168 21.1, at 128 19.0.  One species: R =
-// 4 14.7, 8 9.7.  8 or 16 warps a block in place of 4: 23.8 and 25.3 against 23.2
-// (R = 4, 128 registers).  Loading the next run's cells while the current one
-// is added, into a second register set: 26.3 to 28.6.
+// cells) over more sums; it takes registers from the warps in flight.
+// Columns of every leaf, Nside 1, R = 2 / 4 / 8:
+//   F32-Kahan, 256^3, ms, at 4 blocks (1 species 16.5 / 14.7 / 9.6, 2: 21.0 / 19.2 / 13.1, 4: 29.1 /
+//   21.4 / 18.9, 8: 49.3 / 38.5 / 80.5, spilling), 5 blocks (16.2 / 14.7 / 9.6, 21.0 / 16.1 / 12.0, 29.8
+//   / 21.4 / 22.9) and 3 blocks (8 species 59.7 / 43.8 / 50.7; 4 species at R = 8 21.0);
+//   FP64, 128^3, ms (1 species 7.76 / 7.12 / 7.27, 2: 14.4 / 14.1 / 14.4, 4: 27.8 / 28.0 / 28.6, 8: 55.3 /
+//   55.4 / 55.9; 3 or 5 blocks within 1 %) and 32^3, us (90 / 96 / 118, 134 / 143 / 219, 203 / 255 / 381, 351 /
+//   415 / 567).
+// 8 or 16 warps a block in place of 4: 23.8 and 25.3 against 23.2 ms (256^3, 4 species,
+// R = 4, 128 registers).  Loading the next run's cells while the current one is
+// added, into a second register set: 26.3 to 28.6.
 constexpr int kBeamWarps = 4;
 template <int MODE, int SM>
 __host__ __device__ constexpr int beam_r()
@@ -562,7 +567,7 @@ __host__ __device__ constexpr int beam_blocks()
 {
     if (R == 1) return MODE == RT_MODE_FP64 ? (SM >= 8 ? 3 : SM >= 4 ? 4 : SM >= 2 ? 6 : 8) : (SM >= 8 ? 6 : 8);
     if (MODE == RT_MODE_F32_KAHAN && SM == 4 && R == 4) return 5;
-    return MODE == RT_MODE_FP64 ? (SM >= 8 ? 2 : 4) : (SM >= 8 ? 3 : 4);
+    return MODE == RT_MODE_FP64 ? (SM >= 8 ? 2 : 4) : (SM == 2 ? 5 : 4);
 }
 
 // Leaves a thread takes in the adjoint.  It is launched one direction at a time,

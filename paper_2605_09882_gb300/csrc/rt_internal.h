@@ -58,7 +58,7 @@ struct DevStats {
     unsigned long long exit_fb;
     unsigned long long lookup_fb;
     int status;
-    int gather_off;                // adjoint: nonzero when the leaf-gather form does not apply
+    int gather_off;                // nonzero when the shared-offset form (columns, epilogue, adjoint) did not apply
     long long fault_ray;
     int gathered;                  // set when a leaf-gather adjoint ran
     int pad;
@@ -82,7 +82,7 @@ struct TraceArgs {
     int batch;               // ray groups per queue pop
     int gw;                  // rays a group: 32, or fewer to spread a call of few rays over the warps
     int layout;              // ray order: 0 direction-major (sources padded to 32), 1 source-major
-    int dgroup;              // layout 0: directions per group (a power of two dividing nd; <= 1: one)
+    int dgroup;              // layout 0: directions per group (a divisor of nd; <= 1: one)
     int pair;                // forward on a uniform cube: two rays per lane (k_trace_pair; n_src_pad % 64 == 0)
     // path recording (KIND 3): per 32-ray group, segment k of lane i is entry
     // rec_off[g] + 32 k + i of rec_leaf / rec_ds
