@@ -26,6 +26,7 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
+FP32_OPS_PER_SEGMENT = 4 * 4  # a Kahan step for each of 4 species
 BYTES_PER_SEGMENT = 8 + 1 + 4 * 4  # key + level + 4 FP32 densities (algorithmic)
 NSIDE = 1
 LEVEL = 9
@@ -157,14 +158,15 @@ class Clocks:
                 "samples": len(sm)}
 
 
-def issue_roofline(seg_per_launch, launch_s, clk, hbm_gbs, hbm_kind, dev):
-    """The bound of the trace kernel: instruction issue.  Every SM has four
-    schedulers that issue at most one warp instruction per cycle each, so the
-    issue peak is SMs x 4 x the SM clock (the median sampled under load).
-    achieved = segments/s x warp instructions per segment (ncu, 256^3 capture
-    of the same sources).  Beside it: the effective HBM fraction of the 25
-    algorithmic bytes per segment (above 1 because L2 serves the re-reads) and
-    the fraction of HBM bandwidth the measured DRAM traffic uses."""
+def trace_roofline(seg_per_launch, launch_s, clk, hbm_gbs, hbm_kind, dev):
+    """The bound of the trace kernel: the FP32 pipe.  A segment takes 16 FP32
+    operations at 4 species (a Kahan step is a fused multiply-add, an addition and two
+    subtractions), and an SM does 128 a cycle: the peak is SMs x 128 x the SM
+    clock (the median sampled under load).  Beside it: the issue rate (segments/s x
+    warp instructions per segment, ncu, 256^3 capture of the same sources,
+    against four warp instructions a cycle and SM), the effective HBM fraction
+    of the 25 algorithmic bytes per segment (above 1 because L2 serves the
+    re-reads) and the fraction of HBM bandwidth the measured DRAM traffic uses."""
     import torch
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = (clk or {}).get("sm_mhz") or 2070.0
@@ -172,8 +174,12 @@ def issue_roofline(seg_per_launch, launch_s, clk, hbm_gbs, hbm_kind, dev):
     prof = kernel_profile()
     seg_rate = seg_per_launch / launch_s
     eff = BYTES_PER_SEGMENT * seg_rate / 1e9
-    r = {"bound": "issue", "achieved": None, "peak": issue_peak, "unit": "warp-instructions/s", "frac": None,
-         "traffic": None, "peak_kind": f"derived: {sms} SMs x 4 schedulers x {mhz:.0f} MHz (median under load)",
+    fma_peak = sms * 128 * mhz * 1e6
+    r = {"bound": "fp32", "achieved": seg_rate * FP32_OPS_PER_SEGMENT, "peak": fma_peak, "unit": "FP32 operations/s",
+         "frac": seg_rate * FP32_OPS_PER_SEGMENT / fma_peak,
+         "traffic": None, "peak_kind": f"derived: {sms} SMs x 128 x {mhz:.0f} MHz (median under load)",
+         "fp32_ops_per_segment": FP32_OPS_PER_SEGMENT,
+         "issue": {"achieved": None, "peak": issue_peak, "unit": "warp-instructions/s", "frac": None},
          "warp_inst_per_segment": None, "dram_frac": None,
          "effective_hbm": {"bytes_per_segment": BYTES_PER_SEGMENT, "achieved": eff, "peak": hbm_gbs, "unit": "GB/s",
                            "frac": eff / hbm_gbs, "peak_kind": hbm_kind},
@@ -181,8 +187,8 @@ def issue_roofline(seg_per_launch, launch_s, clk, hbm_gbs, hbm_kind, dev):
          "profile": "profiles/trace_f32k_uniform512.md (256^3 capture, per segment)"}
     if prof is not None:
         r["warp_inst_per_segment"] = prof["warp_inst_per_segment"]
-        r["achieved"] = seg_rate * prof["warp_inst_per_segment"]
-        r["frac"] = r["achieved"] / issue_peak
+        r["issue"]["achieved"] = seg_rate * prof["warp_inst_per_segment"]
+        r["issue"]["frac"] = r["issue"]["achieved"] / issue_peak
         r["traffic"] = prof["dram_bytes_per_segment"] * seg_per_launch
         r["dram_frac"] = r["traffic"] / launch_s / (hbm_gbs * 1e9)
         r["ncu"] = {"issue_active_pct": prof["issue_active_pct"], "lts_hit_pct": prof["lts_hit_pct"],
@@ -685,13 +691,13 @@ def main():
     value = world * seg_per_step * a.steps / (total_ms / 1e3)
     avg_launch_s = float(np.mean(launch_ms)) / 1e3
     peak, peak_kind = peaks()
-    roofline = issue_roofline(seg_per_step, avg_launch_s, clk, peak, peak_kind, dev)
+    roofline = trace_roofline(seg_per_step, avg_launch_s, clk, peak, peak_kind, dev)
 
     extras = {}
     cpu = None
     e2e = None
     if not a.no_extras:
-        # ---- FP64 form (same walk, FP64 columns)
+        # ---- FP64 form (FP64 columns)
         out64 = torch.empty((n, nd, 4), dtype=torch.float64, device=dev)
         fwd("fp64", out64)
         barrier()
@@ -714,11 +720,11 @@ def main():
         dgemm = 2 * 8192 ** 3 / best
         extras["fp64_peak"] = {"dgemm_tflops": dgemm / 1e12,
                                "what": "cuBLAS FP64 GEMM 8192^3 on this GPU (2 N^3 flops, best of 3)"}
-        # the FP64 walk's FP64 operations per segment at 4 species: ds (1),
-        # the column update (4 DMUL + 4 DADD) and one exit-time update (2)
-        extras["fp64_form"]["fp64_ops_per_segment"] = 11
-        extras["fp64_form"]["fp64_ops_per_s"] = 11 * s64["segments"] / t64
-        extras["fp64_form"]["frac_of_dgemm_fma_rate"] = 11 * s64["segments"] / t64 / (dgemm / 2)
+        # its FP64 operations per segment at 4 species: the column update (4 DMUL
+        # + 4 DADD; the lengths come from the step tables)
+        extras["fp64_form"]["fp64_ops_per_segment"] = 8
+        extras["fp64_form"]["fp64_ops_per_s"] = 8 * s64["segments"] / t64
+        extras["fp64_form"]["frac_of_dgemm_fma_rate"] = 8 * s64["segments"] / t64 / (dgemm / 2)
         del A, B
         # agreement of the two forms on the full output
         mx = torch.zeros(4, dtype=torch.float64, device=dev)
@@ -858,7 +864,8 @@ def main():
         "cpu_baseline": cpu,
         "e2e": e2e,
         "clocks": clk,
-        "gpu_launches": 2 * a.steps,  # per step: the density check and the trace
+        # per step: k_beam_ref, k_beam_setup, k_beam_dens, k_beam and k_trace_pair (for left-out sources: none here)
+        "gpu_launches": 5 * a.steps,
     }
     line.update(extras)
     if rank == 0:
