@@ -203,7 +203,8 @@ extern "C" int rt_trace_columns_host(const uint64_t* h_keys, const uint8_t* h_le
             (c >= 2 && cudaStreamWaitEvent(cs, w.ev[3 * (c - 2) + 2], 0) != cudaSuccess))
             return cuda_error(who);
         // (lent tables of no size: the call walks)
-        guard.tree->fwd_tab_bytes = guard.tree->fwd_tab && n >= 32 && beam_vote(h_src + 3 * s0, n, guard.tree->dev.uniform_level) ? w.cap[kTab] : 0;
+        const bool form = guard.tree->fwd_tab && n >= 32 && beam_vote(h_src + 3 * s0, n, guard.tree->dev.uniform_level);
+        guard.tree->fwd_tab_bytes = form ? w.cap[kTab] : 0;
         st = trace_columns_impl(guard.tree, src + 3 * s0, n, nside, dens, S, dens_dtype, mode, slot, stream, false);
         if (st != RT_OK) return st;
         const size_t bytes = (size_t)n * nd * S * osz;
