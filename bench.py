@@ -864,7 +864,7 @@ def main():
         "cpu_baseline": cpu,
         "e2e": e2e,
         "clocks": clk,
-        # per step: k_beam_ref, k_beam_setup, k_beam_dens, k_beam and k_trace_pair (for left-out sources: none here)
+        # per step: k_beam_ref, k_beam_setup, k_beam_dens, k_beam and k_trace (for left-out sources: none here)
         "gpu_launches": 5 * a.steps,
     }
     line.update(extras)

@@ -359,11 +359,11 @@ int rt_set_step_cap(rt_octree* tree, int64_t cap);
  * 0 = default 4; a call too small to give every warp that many takes fewer,
  * and of fewer rays).  Applies to later calls in this process.  The F32-Kahan
  * forward of rt_trace_columns on a full cube of equal-level leaves with FP32
- * densities of 1, 2, 4 or 8 species walks two rays per lane: its warps pop
- * one 64-source block and one direction group at a time, whatever
- * groups_per_pop says, and at most 3 of its blocks fit on an SM.  The form of
- * rt_trace_columns and the adjoint that walks nothing has a launch shape of its
- * own. */
+ * densities of 1, 2 or 4 species and at least 2^24 rays, where it walks, walks two
+ * rays per lane: its warps pop one 64-source block and one direction group at
+ * a time, whatever groups_per_pop says, and at most 3 of its blocks fit on an
+ * SM.  The form of rt_trace_columns and the adjoint that walks nothing has a
+ * launch shape of its own. */
 int rt_set_launch(int threads_per_block, int blocks_per_sm, int groups_per_pop);
 
 /* Caps the coarse-table level of later rt_build_octree calls (-1, the

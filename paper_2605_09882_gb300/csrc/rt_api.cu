@@ -321,10 +321,15 @@ int rt::trace_columns_impl(const rt_octree* t, const double* d_src, int64_t n_sr
         st = check_densities(d_dens, t->dev.n, n_species, a.dens_f64, 0, t->st, s);
         if (st != RT_OK) return st;
     }
-    // leaf centres of a uniform cube share their exit sequences: two rays per
-    // lane (FP32 densities with 1, 2, 4 or 8 species, direction-major order)
-    a.pair = mode == RT_MODE_F32_KAHAN && a.t.uniform_level >= 0 && a.layout == 0 && !a.dens_f64 &&
-             (n_species == 1 || n_species == 2 || n_species == 4 || n_species == 8);
+    // Leaf centres of a uniform cube share their exit sequences: two rays per lane
+    // (FP32 densities with 1, 2 or 4 species, direction-major order) where the
+    // form above does not run (a captured stream, few sources of a large cube) and the
+    // rays fill the chip several times over.  us, two against one: every leaf of
+    // 128^3 (2.5e7 rays) 1 species 2495 / 2745, 4 3167 / 3436, 8 7604 / 5497; a 32nd of
+    // 256^3 (6.3e6) 1226 / 1192, 1442 / 1512, scattered points 5128 / 4230; of 64^3 (9.8e4)
+    // 116 / 34, 76 / 39, scattered 537 / 83; every leaf of 16^3 (4.9e4) 56 / 19, 36 / 21.
+    a.pair = mode == RT_MODE_F32_KAHAN && a.t.uniform_level >= 0 && a.layout == 0 && !a.dens_f64 && !beam.p &&
+             (n_species == 1 || n_species == 2 || n_species == 4) && n_src * a.nd >= (1ll << 24);
     if (a.pair) a.n_src_pad = (n_src + 63) / 64 * 64;
     const int fit = a.pair ? occupancy_pair(n_species, g_block)
                            : occupancy_fwd(0, mode, n_species, a.t.uniform_level >= 0, g_block);

@@ -34,7 +34,6 @@ cudaError_t launch_forward(const TraceArgs& a, int mode, int block, int grid, cu
         case 1: k_trace_pair<1><<<grid, block, 0, s>>>(a); break;
         case 2: k_trace_pair<2><<<grid, block, 0, s>>>(a); break;
         case 4: k_trace_pair<4><<<grid, block, 0, s>>>(a); break;
-        case 8: k_trace_pair<8><<<grid, block, 0, s>>>(a); break;
         default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -84,8 +83,7 @@ int occupancy_pair(int S, int block)
     int n = 0;
     if (S == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace_pair<1>, block, 0);
     else if (S == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace_pair<2>, block, 0);
-    else if (S == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace_pair<4>, block, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace_pair<8>, block, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace_pair<4>, block, 0);
     return n;
 }
 

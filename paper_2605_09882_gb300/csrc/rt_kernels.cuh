@@ -385,8 +385,7 @@ k_trace(const TraceArgs a)
 // unit, a 64-source block and one group of dgroup directions, in the order of
 // k_trace's direction groups; lane i walks sources 64u + i and 64u + 32 + i
 // together for each direction of the group, and one at a time where the two
-// do not qualify.  After the shared-offset form it walks the sources that form
-// left out, one ray a lane.
+// do not qualify.
 #ifndef RT_MIN_BLOCKS_PAIR
 #define RT_MIN_BLOCKS_PAIR 3  // 80 registers: two rays' state without spilling the loop
 #endif
@@ -406,41 +405,19 @@ template <int SM>
 __global__ void __launch_bounds__(256, RT_MIN_BLOCKS_PAIR) k_trace_pair(const TraceArgs a)
 {
     const int lane = threadIdx.x & 31;
-    // after the shared-offset form: the sources it left out, 32 of the list and one
-    // direction a unit
-    const bool rest = a.gate && *(volatile const int*)a.gate == 0;
-    const unsigned n_rest = rest ? *(volatile const unsigned*)a.n_rest : 0u;
-    if (rest && n_rest == 0u) return;
-    const int D = rest || a.dgroup <= 1 ? 1 : a.dgroup;
-    const unsigned long long nb = rest ? (n_rest + 31u) >> 5 : (unsigned long long)a.n_src_pad >> 6;
-    const unsigned long long units = nb * (unsigned long long)(a.nd / D);
+    const int D = a.dgroup > 1 ? a.dgroup : 1;
+    const unsigned long long nb2 = (unsigned long long)a.n_src_pad >> 6;
+    const unsigned long long units = nb2 * (unsigned long long)(a.nd / D);
     const long long cap = a.t.step_cap;
     unsigned long long n_rays = 0, n_segs = 0, n_efb = 0, n_lfb = 0;
-    // A warp's first unit goes by its number, and the queue hands out the rest: the
-    // warps of a block take neighbouring units, whatever the order in which they
-    // arrive, and fewer units than blocks go to as many SMs.  64^3, 16384 scattered
-    // points, us for 1 / 4 species: first units from the queue 602 / 372 (476 with
-    // 4 once the gate delays the warps), by number 559 / 345; 33 sources, Nside 2,
-    // one unit a block 379, neighbouring 412.
-    const unsigned long long warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const unsigned long long mine = units <= gridDim.x ? warp * gridDim.x + blockIdx.x : blockIdx.x * wpb + warp;
-    for (bool first = true;; first = false) {
-        unsigned long long u = mine;
-        if (!first && lane == 0) u = gridDim.x * wpb + atomicAdd(&a.st->queue, 1ull);
+    for (;;) {
+        unsigned long long u = 0;
+        if (lane == 0) u = atomicAdd(&a.st->queue, 1ull);
         u = __shfl_sync(RT_FULL, u, 0);
         if (u >= units) break;
-        const unsigned long long gg = u / nb, bp = u - gg * nb;
-        long long s0, s1;
-        if (rest) {
-            const unsigned long long i = (bp << 5) + lane;  // 32 of the list and one direction
-            if (i >= n_rest) continue;
-            s0 = (long long)__ldg(a.rest + i);
-            s1 = a.n_src;
-        } else {
-            s0 = (long long)(bp << 6) + lane;
-            s1 = s0 + 32;
-            if (s0 >= a.n_src) continue;
-        }
+        const unsigned long long gg = u / nb2, bp = u - gg * nb2;
+        const long long s0 = (long long)(bp << 6) + lane, s1 = s0 + 32;
+        if (s0 >= a.n_src) continue;
         const bool two = s1 < a.n_src;
         for (int dd = 0; dd < D; dd++) {
             const int q = (int)gg * D + dd;
