@@ -132,8 +132,8 @@ int rt_healpix_dirs(int nside, double* h_out);
  * for example) take no walk: every ray of a direction has the same steps, and
  * the columns are summed from step tables and a row-ordered copy of the
  * densities, bit for bit those of the walk.  At least a sixteenth of the leaves
- * must have a source; RT_MODE_FP64 asks for most of each 32^3-leaf block and at
- * least 2^18 rays.  The sources are checked on the device; those elsewhere (all, if
+ * must have a source, most of each 32^3-leaf block, and there must be at least
+ * 2^18 rays.  The sources are checked on the device; those elsewhere (all, if
  * over a sixteenth of them) are walked.
  * Memory: every call of that shape, whatever its sources turn out to be, takes
  * two copies of the densities (n_leaves x 1, 2, 4 or 8 values each) and a

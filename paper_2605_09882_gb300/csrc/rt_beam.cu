@@ -994,26 +994,27 @@ static long long beam_blocks_of(int L, int64_t n_src)
     return std::min<long long>(1ll << (3 * (L - 5)), (n_src + 32767) / 32768 + 1);
 }
 
-// True where the form pays, us of it and of the walk, sources at leaf centres.
+// True where the form pays, us of it and of the walk (one ray a lane), sources at leaf
+// centres.  It computes whole 32^3 blocks: at most 1.5 leaves computed a source
+// (FP64, bound by its operations: 1 species 2, 5 to 8 species 1.2), and 2^18 rays to
+// fill the chip.
 //
-// F32-Kahan: sources in a sixteenth of the leaves or more: 4 species, an eighth of
-// a 32^3 cube 45 / 59, a sixteenth 45 / 57; of 64^3 78 / 102, of 256^3 1408 / 3086.  It
-// gains below that too (256^3, a 64th: 520 / 805), but scattered points
-// pay for the vote (12 us), of which a smaller call is a larger part.
+// F32-Kahan, 64^3 at 1.25, 1.5 and 2 leaves a source: 1 species 97 / 153, 81 / 100, 69 /
+// 60; 4 species 130 / 186, 95 / 111, 88 / 65; 8 species 172 / 294, 124 / 168, 97 / 93.
+// Every leaf of 32^3 (3.9e5 rays) 54 / 41, 58 / 49, 63 / 67, half of it 53 / 34, 57 / 40, 63 / 47.
+// FP64, the same: 381 / 731, 246 / 404, 190 / 235; 1252 / 1445, 782 / 827, 544 / 528;
+// 2430 / 2393, 1501 / 1261, 1041 / 1041.  32^3, 1 species: 92 / 88 on densities in
+// L2, 95 / 122 on new ones, half of it (2.0e5) 92 / 72, at Nside 2 203 / 280.
 //
-// FP64 is bound by its FP64 operations in both forms, and this one computes whole
-// 32^3 blocks: at most 1.5 leaves computed a source (5 to 8 species: 1.2), and enough
-// rays to fill the chip.  64^3 at 1.25, 1.5 and 2 leaves a source: 1 species 381 /
-// 731, 246 / 404, 190 / 235; 4 species 1252 / 1445, 782 / 827, 544 / 528; 8 species
-// 2430 / 2393, 1501 / 1261, 1041 / 1041.  32^3, 1 species, every leaf (3.9e5 rays): 92 /
-// 88 on densities in L2, 95 / 122 on new ones; half of them (2.0e5) 92 / 72 and
-// 203 / 280 at Nside 2, a quarter 92 / 61 and 201 / 156.
+// Sources in a sixteenth of the leaves or more: of 128^3, 4 species, F32-Kahan, 191 / 266, of
+// 256^3 1408 / 3086.  It gains below that too (256^3, a 32nd 813 / 1512), but scattered
+// points pay for the vote (12 us), of which a smaller call is a larger part.
 static bool beam_pays(int L, int64_t n_src, int nd, int S, int mode, int64_t n_leaves)
 {
-    if (n_src * 16 < n_leaves) return false;
-    if (mode != RT_MODE_FP64) return true;
     const long long done = beam_blocks_of(L, n_src) * 32768;
-    return n_src * nd >= (1ll << 18) && (S > 4 ? done * 5 <= n_src * 6 : done * 2 <= n_src * 3);
+    if (n_src * 16 < n_leaves || n_src * nd < (1ll << 18)) return false;
+    if (mode != RT_MODE_FP64 || (S > 1 && S <= 4)) return done * 2 <= n_src * 3;
+    return S == 1 ? done <= n_src * 2 : done * 5 <= n_src * 6;
 }
 
 // Bytes of tables the shared-offset trace keeps on this octree, 0 when its

@@ -168,11 +168,12 @@ def test_host_call_on_cubes(rt):
         cubes[level] = keys, lev, dict(centres=centres, offset=centres + np.array([7, -11, 3]) * h / 32, half=half, moved=moved,
                                        scattered=rng.random(centres.shape))
     n6 = 1 << 18
-    calls = [(6, 2, 1, "f32k", "centres", n6 // 5), (6, 2, 1, "f32k", "centres", n6 // 5), (6, 3, 1, "f32k", "centres", 0),
-             (6, 8, 1, "f32k", "offset", n6 // 3), (6, 2, 1, "f32k", "centres", n6 - 64), (6, 1, 2, "fp64", "centres", 0),
-             (5, 4, 2, "f32k", "centres", 0), (5, 4, 1, "f32k", "offset", 4096), (5, 4, 2, "fp64", "offset", 32768),
-             (5, 4, 1, "f32k", "centres", 4096), (6, 2, 1, "f32k", "half", 0), (6, 2, 1, "f32k", "moved", n6 // 4),
-             (5, 2, 1, "f32k", "scattered", 0), (6, 2, 4, "f32k", "centres", 0), (5, 1, 1, "f32k", "centres", 1 << 14)]
+    n5 = 1 << 15
+    calls = [(6, 2, 1, "f32k", "centres", n6 // 3), (6, 2, 1, "f32k", "centres", n6 // 3), (6, 3, 1, "f32k", "centres", n6 // 4),
+             (6, 8, 1, "f32k", "offset", n6 // 3), (6, 2, 1, "f32k", "centres", n6 - 64), (6, 1, 2, "fp64", "centres", n6 // 4),
+             (5, 4, 2, "f32k", "centres", n5), (5, 4, 1, "f32k", "offset", n5), (5, 4, 2, "fp64", "offset", n5),
+             (5, 4, 1, "f32k", "centres", 4096), (6, 2, 1, "f32k", "half", n6 // 4), (6, 2, 1, "f32k", "moved", n6 // 4),
+             (5, 2, 1, "f32k", "scattered", n5), (6, 2, 4, "f32k", "centres", n6 // 2), (5, 1, 1, "f32k", "centres", 0)]
     rt.trace_columns_host_release()
     for level, S, nside, mode, how, chunk in calls:
         keys, lev, sources = cubes[level]
