@@ -890,7 +890,7 @@ static BeamScratch beam_scratch(char* p, char* v, int nd, int L, int64_t n_src, 
     const size_t steps = adjoint ? (size_t)nd * lcap : 0;
     const size_t bytes[] = {sizeof(BeamRef), (size_t)nd * sizeof(int4), (size_t)nd * lcap * rsz, (size_t)nd * lcap * 4,
                             (size_t)nd * 3 * pcap * 4, (size_t)nd * 3 * pcap * 4, steps * 4,
-                            steps * (mode == RT_MODE_FP64 ? 8 : 4), (size_t)(adjoint ? nd : 2) * 8};
+                            steps * (mode == RT_MODE_FP64 ? 8 : 4), (size_t)(adjoint ? nd : 1) * 8};
     size_t at[10] = {0};
     for (int i = 0; i < 9; i++) at[i + 1] = at[i] + round256(bytes[i]);
     b.most = (unsigned int)(n_src / 16);
@@ -1167,7 +1167,7 @@ int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check,
     g.dgroup = a.dgroup > 1 ? a.dgroup : 1;
     g.blocks = beam_blocks_of(L, a.n_src);
     const int op = epilogue ? kBeamEpilogue : kBeamColumns;
-    cudaError_t e = beam_setup(a, mode, b, b.most, 2, s);
+    cudaError_t e = beam_setup(a, mode, b, b.most, 1, s);
     if (e == cudaSuccess) {
         if (mode == RT_MODE_FP64)
             e = SM == 1 ? go_trace<RT_MODE_FP64, 1>(g, rows, check, op, s) : SM == 2 ? go_trace<RT_MODE_FP64, 2>(g, rows, check, op, s)
@@ -1180,7 +1180,6 @@ int launch_beam(rt_octree* t, TraceArgs& a, int mode, bool epilogue, bool check,
     a.gate = &t->st->gather_off;
     a.rest = b.rest;
     a.n_rest = &b.ref->n_rest;
-    a.rest_queue = b.queue + 1;
     return RT_OK;
 }
 

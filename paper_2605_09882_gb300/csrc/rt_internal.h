@@ -101,7 +101,6 @@ struct TraceArgs {
     // when *gate is zero (NULL: none)
     const uint32_t* rest;
     const unsigned int* n_rest;
-    unsigned long long* rest_queue;  // rays of theirs handed out so far by k_trace
 };
 
 // Ray order of a trace: direction-major (32 neighbouring sources share a

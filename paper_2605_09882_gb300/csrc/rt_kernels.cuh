@@ -254,29 +254,22 @@ k_trace(const TraceArgs a)
     unsigned long long total = (unsigned long long)(a.layout ? a.n_src : a.n_src_pad) * (unsigned long long)a.nd;
     const long long cap = a.t.step_cap;
     unsigned long long n_rays = 0, n_segs = 0, n_efb = 0, n_lfb = 0;
-    bool gated = GATED, rest = false;
+    bool rest = false;
     unsigned long long rest_pad = 0;
+    if (GATED && *(volatile const int*)a.gate == 0) {
+        // the shared-offset form ran before: only the sources it left out, if any
+        const unsigned n = *(volatile const unsigned*)a.n_rest;
+        if (n == 0u) return;
+        rest = true;
+        rest_pad = (n + 31u) & ~31u;
+        total = rest_pad * (unsigned long long)a.nd;
+    }
+    // (the left-out sources are few: a group a pop; 32^3, FP64, 4 species, one source
+    // in 32 left out: 514 -> 375 us, 64^3 3210 -> 2358)
+    const int batch = rest ? 1 : a.batch;
     for (;;) {
         unsigned long long base = 0;
-        // (the left-out sources are few: a group a pop; 32^3, FP64, 4 species, one source
-        // in 32 left out: 514 -> 375 us, 64^3 3210 -> 2358)
-        const int batch = rest ? 1 : a.batch;
-        if (lane == 0) base = atomicAdd(rest ? a.rest_queue : &a.st->queue, (unsigned long long)gw * (unsigned)batch);
-        if (gated) {
-            // read after the first pop: warps that wait for it first pop in a shuffled
-            // order, which spreads neighbouring groups over the chip (64^3, 65536
-            // scattered points, FP64: 693 us in place of 660)
-            gated = false;
-            if (*(volatile const int*)a.gate == 0) {
-                // the shared-offset form ran before: only the sources it left out, if any
-                const unsigned n = *(volatile const unsigned*)a.n_rest;
-                if (n == 0u) return;
-                rest = true;
-                rest_pad = (n + 31u) & ~31u;
-                total = rest_pad * (unsigned long long)a.nd;
-                continue;
-            }
-        }
+        if (lane == 0) base = atomicAdd(&a.st->queue, (unsigned long long)gw * (unsigned)batch);
         base = __shfl_sync(RT_FULL, base, 0);
         if (base >= total) break;
         for (int kk = 0; kk < batch; kk++) {
